@@ -38,9 +38,9 @@ struct nsli_solver {
     int storage = NSLI_F32;
     long long m = 0, n = 0, ld = 0;
     int elem_bytes = 4, epv = 4, row_bytes = 0, nv = 0;
-    int vpt = 1, consumers = 32, R = 1, nstage = 2, stage_stride = 0;
+    int vpt = 1, R = 1, nstage = 2, stage_stride = 0;
+    int team_warps = 1, teams = 1, ring_offset = 0;   // register-resident rows
     int cluster = 0, slice_nv = 0, cluster_vpt = 0, cluster_lag = 1, cluster_rg = 1;   // long rows on clusters
-    bool guard = true;
     size_t smem = 0;
     int G = 1, red_grid = 1, num_sms = 1;
     long long rows_base = 0;
@@ -82,6 +82,12 @@ struct nsli_solver {
     bool resident = false;
     size_t res_smem = 0;
     int *res_rows = nullptr, *res_cols = nullptr;
+
+    // whole iterations in one launch (iterate_kernel)
+    unsigned int *iter_sync = nullptr;
+    unsigned long long *iter_dmax = nullptr;
+    void *iter_stats = nullptr;
+    bool iter_ok = false;
 
     // row-sharded runs (nsli_shard_*): partial sums of the exchange step
     double *shard_dx = nullptr;
@@ -141,7 +147,7 @@ void free_all(nsli_solver *h)
                    h->dtmp, h->scale, h->part_stat, h->st, h->ver, h->flags,
                    (h->x64 != h->x) ? (void *)h->x64 : nullptr,
                    (h->n2_meta != h->n2_64) ? (void *)h->n2_meta : nullptr,
-                   h->rp, h->cp, h->ci, h->ri, h->row_cnt, h->col_cnt, h->row_pieces, h->col_pieces,
+                   h->rp, h->cp, h->ci, h->ri, h->row_cnt, h->col_cnt, h->row_pieces, h->col_pieces, h->iter_sync, h->iter_dmax, h->iter_stats,
                    h->va, h->vc, h->coef, h->row_slots, h->col_slots, h->res_rows, h->res_cols, h->rtab};
     for (void *p : dev)
         if (p)
@@ -156,8 +162,66 @@ void free_all(nsli_solver *h)
         cudaStreamDestroy(h->stream);
 }
 
-// Launch shape of the Map kernel (see nsli_kernels.cu): rows are padded to
-// whole 16-byte vectors; each consumer thread owns vpt vectors of every row.
+// Launch shape of the Map of register-resident rows (nsli_dense.cu).
+int choose_teams(nsli_solver *h, bool pooled)
+{
+    const bool f64 = h->storage == NSLI_F64;
+    const int vlim = map_vpt_limit(h->storage), acc_bytes = f64 ? 8 : 4;
+    h->G = (int)std::min<long long>(h->num_sms, h->m);
+    h->rows_base = h->m / h->G;
+    h->rows_rem = (int)(h->m % h->G);
+    const long long rows = h->rows_base + (h->rows_rem ? 1 : 0);
+    // One team with one vector per thread where a CTA's block is a group or
+    // two (up to 16 rows): the rows of a group go side by side anyway, and
+    // there are no teams' y to add (an iteration of 2000 x 500 binary32: 8.20
+    // us, with 16 one-warp teams 8.25 us).  Also short rows of a pool (below
+    // 2048 entries), whose items of hundreds of rows are summed row after row:
+    // the iterate of such a problem moves by 1 / n a step, so that another
+    // order of the sums would show in its tenth digit (1.3e-9 at n = 1024).
+    const bool one_team = h->nv <= kMapMaxConsumers && (rows <= 16 || (pooled && h->n < 2048));
+    // Otherwise as many vectors per thread as the registers hold (few warps
+    // then share a row, and meet), fewer only where one warp holds the row
+    // with them: a row takes team_warps warps, and the CTA's 16 mapping warps
+    // hold as many teams as fit.
+    h->vpt = 1;
+    while (!one_team && h->vpt < vlim && h->nv > 32 * h->vpt)
+        h->vpt *= 2;
+    h->team_warps = (h->nv + 32 * h->vpt - 1) / (32 * h->vpt);
+    h->teams = one_team ? 1 : (kMapMaxConsumers / 32) / h->team_warps;
+    // with several teams: an area that stages x and adds the teams' y
+    const long long xbytes = (long long)h->ld * acc_bytes;
+    const long long ybytes = (long long)(h->teams / 2) * h->team_warps * 32 * h->vpt * h->epv * acc_bytes;
+    h->ring_offset = kTeamHeader + (h->teams > 1 ? (int)round_up(std::max(xbytes, ybytes), 128) : 0);
+    // Rows per ring slot (a slot is one row group): as many as the instance
+    // takes (the fixed cost of a group is shared by its rows) while the ring
+    // holds a slot in use per team and one more (large teams, which refill a
+    // group later: twice as many and one more), and while every team of a
+    // small block gets rows.  Measured per iteration: 8192 x 2048 binary32,
+    // eight teams: two rows 17.4 us, one 21.1 us; Map of 32768 x 8192 bf16, two
+    // teams: one row 145 us, two 96 us.
+    const int budget = kSmemMax - h->ring_offset;
+    auto stride_of = [&](int r) { return (int)round_up((long long)r * (h->row_bytes + 32), 128); };
+    const int least = h->team_warps >= kLargeTeam ? 2 * h->teams + 1 : h->teams + 1;
+    h->R = 1;
+    for (int r = one_team ? team_rg_max(1, f64) : std::min(4, team_rg_max(h->vpt, f64)); r > 1; r /= 2)
+        if (budget / stride_of(r) >= least && (one_team || rows >= (long long)r * h->teams)) {
+            h->R = r;
+            break;
+        }
+    h->stage_stride = stride_of(h->R);
+    h->nstage = std::min(kMapMaxStages, budget / h->stage_stride);
+    if (h->nstage < h->teams + 1)
+        return set_err(h, NSLI_ERR_UNSUPPORTED, "row does not fit the shared-memory ring");
+    if (!pooled)   // a block that fits needs no more stages than it has slots
+        h->nstage = (int)std::min<long long>(h->nstage, (rows + h->R - 1) / h->R);
+    h->smem = (size_t)h->ring_offset + (size_t)h->nstage * h->stage_stride;
+    h->red_grid = (int)((h->ld + kReduceCols - 1) / kReduceCols);
+    return NSLI_OK;
+}
+
+// Layout and launch shape: rows are padded to whole 16-byte vectors; each
+// mapping thread owns vpt vectors of every row (0: rows longer than the
+// registers hold).
 int choose_config(nsli_solver *h)
 {
     switch (h->storage) {
@@ -171,13 +235,7 @@ int choose_config(nsli_solver *h)
     h->row_bytes = (int)(h->ld * h->elem_bytes);
     h->nv = h->row_bytes / 16;
     const int vlim = map_vpt_limit(h->storage);
-    h->vpt = 0;
-    for (int v = 1; v <= vlim; v *= 2) {
-        if ((h->nv + v - 1) / v <= kMapMaxConsumers) {
-            h->vpt = v;
-            break;
-        }
-    }
+    h->vpt = h->nv <= vlim * kMapMaxConsumers ? vlim : 0;
     if (h->vpt == 0) {
         // long rows: thread-block clusters that split the columns
         // (NSLI_LONG_CLUSTER=0 selects the two-pass kernel): the fewest CTAs
@@ -242,8 +300,6 @@ int choose_config(nsli_solver *h)
                         if (v >= 1 && v <= 3 && v <= ng - 2)
                             h->cluster_lag = v;
                     }
-                    h->consumers = kMapMaxConsumers;
-                    h->guard = true;
                     h->nstage = ns;
                     h->stage_stride = stride;
                     h->R = 1;
@@ -263,8 +319,6 @@ int choose_config(nsli_solver *h)
         // n = 54000: four rows per group beat fewer even where part of them
         // must come back from DRAM); the partial-sum row goes to shared
         // memory when it fits in 220 KB.
-        h->consumers = 512;
-        h->guard = true;
         h->nstage = 0;
         h->stage_stride = 0;
         h->G = (int)std::min<long long>(h->num_sms, h->m);
@@ -284,28 +338,7 @@ int choose_config(nsli_solver *h)
         h->red_grid = (int)((h->ld + kReduceCols - 1) / kReduceCols);
         return NSLI_OK;
     }
-    h->consumers = (int)round_up((h->nv + h->vpt - 1) / h->vpt, 32);
-    // bytes of A per ring slot: 64 KiB unless NSLI_MAP_SLOT_KB (4..96) overrides it
-    int slot_target = 65536;
-    if (const char *env = std::getenv("NSLI_MAP_SLOT_KB")) {
-        const int kb = std::atoi(env);
-        if (kb >= 4 && kb <= 96)
-            slot_target = kb * 1024;
-    }
-    h->guard = (long long)h->consumers * h->vpt != h->nv;
-    const int rg = map_rows_per_group(h->vpt, h->storage == NSLI_F64 ? 8 : 4);
-    h->R = rg * std::max(1, std::min(64 / rg, slot_target / (h->row_bytes * rg)));
-    h->stage_stride = (int)round_up((long long)h->R * h->row_bytes + (long long)h->R * 32, 128);
-    const int budget = 232448 - kSmemHeader;
-    h->nstage = std::min(8, budget / h->stage_stride);
-    if (h->nstage < 2)
-        return set_err(h, NSLI_ERR_UNSUPPORTED, "row does not fit two shared-memory stages");
-    h->smem = (size_t)kSmemHeader + (size_t)h->nstage * h->stage_stride;
-    h->G = (int)std::min<long long>(h->num_sms, h->m);
-    h->rows_base = h->m / h->G;
-    h->rows_rem = (int)(h->m % h->G);
-    h->red_grid = (int)((h->ld + kReduceCols - 1) / kReduceCols);
-    return NSLI_OK;
+    return choose_teams(h, false);
 }
 
 MapArgs map_args(nsli_solver *h)
@@ -333,6 +366,9 @@ MapArgs map_args(nsli_solver *h)
     a.cluster_vpt = h->cluster_vpt;
     a.cluster_lag = h->cluster_lag;
     a.cluster_rg = h->cluster_rg;
+    a.team_warps = h->team_warps;
+    a.teams = h->teams;
+    a.ring_offset = h->ring_offset;
     return a;
 }
 
@@ -369,10 +405,39 @@ cudaError_t launch_iteration(nsli_solver *h, int rule)
             e = sparse_step_launch(f64, h->stream, h->sp);
         return e;
     }
-    cudaError_t e = map_launch(h->storage, h->vpt, h->guard, h->G, h->consumers, h->smem, h->stream, map_args(h));
+    cudaError_t e = map_launch(h->storage, h->vpt, h->G, h->smem, h->stream, map_args(h));
     if (e != cudaSuccess)
         return e;
     return reduce_launch(h->storage == NSLI_F64, h->red_grid, h->stream, reduce_args(h));
+}
+
+// Iterations per launch of the one-launch form, 0 where it is not taken: the
+// caller asks for graphs of block_iters iterations, the rows are long or
+// sparse, or the stream is being captured.  A launch reads at most about 64
+// GB of A (some 10 ms), so that other streams get their turn and a solve its
+// polls; small systems take up to 1024 iterations.
+int iterations_per_launch(const nsli_solver *h, const nsli_params *p)
+{
+    if (!h->iter_ok || p->block_iters > 0)
+        return 0;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
+        return 0;
+    const long long bytes = h->m * (long long)h->row_bytes;
+    return (int)std::max<long long>(32, std::min<long long>(1024, (64ll << 30) / bytes));
+}
+
+cudaError_t launch_iterations(nsli_solver *h, int iters)
+{
+    IterArgs a;
+    a.map = map_args(h);
+    a.red = reduce_args(h);
+    a.sync = h->iter_sync;
+    a.dmax = h->iter_dmax;
+    a.stats = h->iter_stats;
+    a.iters = iters;
+    a.nblk = h->red_grid;
+    return iterate_launch(h->storage, h->vpt, h->G, h->smem, h->stream, a);
 }
 
 int ensure_graph(nsli_solver *h, int iters, int rule)
@@ -518,6 +583,7 @@ int begin_run(nsli_solver *h, const nsli_params *p, int stop, long long max_iter
     const bool fill = h->rtab && !(h->rtab_lambda == p->lambda);
     b.rtab = fill ? h->rtab : nullptr;
     b.rtab_m = h->m;
+    b.sync = h->iter_sync;
     CK(state_begin_launch(h->stream, h->st, b), "begin run");
     if (fill)
         h->rtab_lambda = p->lambda;
@@ -620,7 +686,10 @@ int nsli_create(nsli_handle *out, int64_t m, int64_t n, int32_t storage, int32_t
     CKC(cudaMalloc(&h->part_y, (size_t)h->G * h->ld * accb), "allocate partial sums");
     CKC(cudaMalloc((void **)&h->part_stat, (size_t)h->G * sizeof(PartStat)), "allocate partial stats");
     CKC(cudaMalloc((void **)&h->rtab, (size_t)(m + 1) * 8), "allocate step table");
-    CKC(cudaMalloc((void **)&h->part_dx, (size_t)h->red_grid * 8), "allocate step partials");
+    CKC(cudaMalloc((void **)&h->part_dx, (size_t)2 * h->red_grid * 8), "allocate step partials");
+    CKC(cudaMalloc((void **)&h->iter_sync, 4 * sizeof(unsigned int)), "allocate grid counters");
+    CKC(cudaMalloc((void **)&h->iter_dmax, (size_t)h->red_grid * 8), "allocate step maxima");
+    CKC(cudaMalloc(&h->iter_stats, (size_t)2 * h->G * 32), "allocate iteration records");
     CKC(cudaMalloc((void **)&h->ybuf, (size_t)h->ld * 8), "allocate y");
     CKC(cudaMalloc((void **)&h->dtmp, (size_t)std::max<long long>(m, h->ld) * 8), "allocate staging");
     CKC(cudaMalloc((void **)&h->st, sizeof(DevState)), "allocate state");
@@ -735,8 +804,14 @@ int nsli_create(nsli_handle *out, int64_t m, int64_t n, int32_t storage, int32_t
         return fail(cuda_err(h, err, "prepare A"));
     if ((rc = read_flags(h)) != NSLI_OK)
         return fail(rc);
-    if (h->cluster == 0)
-        CKC(map_prepare(storage, h->vpt, h->guard, h->smem), "configure Map kernel");
+    if (h->vpt > 0) {
+        int coop = 0, bps = 0;
+        CKC(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device), "cooperative launches");
+        CKC(team_prepare(storage, h->vpt, h->R, team_threads(h->teams, h->team_warps), &bps), "configure Map kernel");
+        h->iter_ok = coop && bps >= 1;
+    }
+    if (h->vpt == 0 && h->cluster == 0)
+        CKC(long_prepare(storage, h->smem), "configure Map kernel");
 #undef CKC
     *out = h;
     return NSLI_OK;
@@ -1227,6 +1302,13 @@ int nsli_iterate(nsli_handle h, const nsli_params *p, int64_t n_iter)
         }
         return NSLI_OK;
     }
+    if (const int per_launch = iterations_per_launch(h, p)) {
+        for (long long done = 0; done < n_iter; done += per_launch) {
+            CK(launch_iterations(h, (int)std::min<long long>(per_launch, n_iter - done)), "launch iterations");
+            h->launches += 1;
+        }
+        return NSLI_OK;
+    }
     const int B = p->block_iters > 0 ? p->block_iters : 32;
     const long long full = n_iter / B;
     const long long rem = n_iter % B;
@@ -1272,8 +1354,7 @@ int nsli_iterate_timed(nsli_handle h, const nsli_params *p, int64_t n_iter, doub
             if (h->sparse)
                 err = sparse_row_launch(h->storage == NSLI_F64, h->stream, h->sp);
             else
-                err = map_launch(h->storage, h->vpt, h->guard, h->G, h->consumers, h->smem, h->stream,
-                                 map_args(h));
+                err = map_launch(h->storage, h->vpt, h->G, h->smem, h->stream, map_args(h));
             if (err != cudaSuccess)
                 break;
             cudaEventRecord(ev[3 * i + 1], h->stream);
@@ -1314,8 +1395,9 @@ int nsli_solve(nsli_handle h, const nsli_params *p, nsli_result *out)
         return rc;
     if ((rc = begin_run(h, p, p->stop, p->max_iter)) != NSLI_OK)
         return rc;
-    const int B = p->block_iters > 0 ? p->block_iters : (h->resident ? kResBlock : 32);
-    if (!h->resident && (rc = ensure_graph(h, B, p->rule)) != NSLI_OK)
+    const int per_launch = iterations_per_launch(h, p);
+    const int B = p->block_iters > 0 ? p->block_iters : (h->resident ? kResBlock : (per_launch ? per_launch : 32));
+    if (!h->resident && !per_launch && (rc = ensure_graph(h, B, p->rule)) != NSLI_OK)
         return rc;
     const int per = launches_per_iteration(h, p->rule);
     int status = NSLI_NOT_CONVERGED;
@@ -1328,6 +1410,9 @@ int nsli_solve(nsli_handle h, const nsli_params *p, nsli_result *out)
         if (h->resident) {
             CK(sparse_resident_launch(h->storage == NSLI_F64, h->stream, h->sp, h->res_smem, B),
                "launch one-CTA iterations");
+            h->launches += 1;
+        } else if (per_launch) {
+            CK(launch_iterations(h, B), "launch iterations");
             h->launches += 1;
         } else {
             CK(cudaGraphLaunch(h->graph, h->stream), "launch iteration graph");
@@ -1406,7 +1491,7 @@ int nsli_map_reduce(nsli_handle h, double *y, int64_t *violated, double *stats)
     } else {
         MapArgs ma = map_args(h);
         ma.ignore_done = 1;  // also after a finished run
-        CK(map_launch(h->storage, h->vpt, h->guard, h->G, h->consumers, h->smem, h->stream, ma), "launch Map");
+        CK(map_launch(h->storage, h->vpt, h->G, h->smem, h->stream, ma), "launch Map");
         CK(reduce_only_launch(h->storage == NSLI_F64, h->red_grid, h->stream, reduce_args(h), h->ybuf),
            "launch Reduce");
     }
@@ -1459,7 +1544,7 @@ int nsli_test_inject_timeout(nsli_handle h, int32_t slot)
     ma.ignore_done = 1;
     ma.skip_slot = slot;
     CK(cudaMemsetAsync(&h->st->error, 0, sizeof(int), h->stream), "clear error");
-    CK(map_launch(h->storage, h->vpt, h->guard, h->G, h->consumers, h->smem, h->stream, ma), "launch Map");
+    CK(map_launch(h->storage, h->vpt, h->G, h->smem, h->stream, ma), "launch Map");
     h->launches += 1;
     int rc = read_state(h);
     CK(cudaMemsetAsync(&h->st->error, 0, sizeof(int), h->stream), "clear error");
@@ -1551,7 +1636,7 @@ int nsli_shard_map(nsli_handle h, double *record)
     } else {
         MapArgs ma = map_args(h);
         ma.ignore_done = 1;
-        CK(map_launch(h->storage, h->vpt, h->guard, h->G, h->consumers, h->smem, h->stream, ma), "launch Map");
+        CK(map_launch(h->storage, h->vpt, h->G, h->smem, h->stream, ma), "launch Map");
         CK(reduce_only_launch(h->storage == NSLI_F64, h->red_grid, h->stream, reduce_args(h), h->ybuf),
            "launch local Reduce");
     }
@@ -1689,7 +1774,7 @@ int rebuild_tables(nsli_pool p)
     std::vector<GroupItem> items;
     std::vector<GroupRed> reds;
     p->live_order.clear();
-    size_t smem = kSmemHeader;
+    size_t smem = kTeamHeader;
     for (size_t sid = 0; sid < p->slots.size(); ++sid) {
         nsli_solver *h = p->slots[sid];
         if (!h)
@@ -1700,7 +1785,6 @@ int rebuild_tables(nsli_pool p)
         gp.map = map_args(h);
         gp.red = reduce_args(h);
         gp.red.G = nitems;
-        gp.nt = h->consumers;
         gp.vpt = h->vpt;
         gp.red_blocks = h->red_grid;
         gp.first_red = (int)reds.size();
@@ -1720,13 +1804,9 @@ int rebuild_tables(nsli_pool p)
     // The persistent launch takes the items in table order from a shared
     // counter: longest first (list scheduling by longest processing time),
     // so the long items start early and the short ones fill the end of the
-    // phase.  An item's time is estimated as its bytes of A over the share
-    // of the CTA's threads its rows occupy.  Which CTA maps an item changes
-    // no result.
+    // phase (by their bytes of A).  Which CTA maps an item changes no result.
     auto est = [&probs](const GroupItem &it) {
-        const GroupProblem &gp = probs[it.prob];
-        return (double)(it.row_end - it.row_begin) * (double)gp.map.row_bytes * (double)kMapMaxConsumers /
-               (double)std::max(1, gp.nt);
+        return (double)(it.row_end - it.row_begin) * (double)probs[it.prob].map.row_bytes;
     };
     std::stable_sort(items.begin(), items.end(),
                      [&est](const GroupItem &a, const GroupItem &b) { return est(a) > est(b); });
@@ -1747,7 +1827,7 @@ int rebuild_tables(nsli_pool p)
             "upload reduce table");
     }
     if (smem > p->smem) {
-        PCK(map_group_prepare(p->storage, smem), "configure grouped Map");
+        PCK(map_group_prepare(p->storage), "configure grouped Map");
         p->smem = smem;
     }
     p->n_items = (int)items.size();
@@ -1842,7 +1922,7 @@ int nsli_pool_add(nsli_pool p, int64_t m, int64_t n, const float *A, int64_t lda
         return perr(p, NSLI_ERR_UNSUPPORTED, "the pool serves rows up to the register-resident limit");
     }
     // control state of the problem's run
-    if ((rc = validate_params(h, prm)) != NSLI_OK || (rc = begin_run(h, prm, prm->stop, prm->max_iter)) != NSLI_OK) {
+    if ((rc = choose_teams(h, true)) != NSLI_OK || (rc = validate_params(h, prm)) != NSLI_OK || (rc = begin_run(h, prm, prm->stop, prm->max_iter)) != NSLI_OK) {
         h->stream = nullptr;
         free_all(h);
         delete h;

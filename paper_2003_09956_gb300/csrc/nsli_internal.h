@@ -99,6 +99,10 @@ struct MapArgs {
     int cluster_vpt;       // ... vectors per thread (instance of the cluster kernel)
     int cluster_lag;       // ... row groups between a group's Map and the wait for its exchange (1..3)
     int cluster_rg;        // ... rows per group (1, or 2 for bf16 / FP8)
+    // register-resident rows (nsli_dense.cu)
+    int team_warps;        // warps that share a row
+    int teams;             // such teams per CTA
+    int ring_offset;       // byte offset of the ring in shared memory
 };
 
 struct ReduceArgs {
@@ -114,12 +118,22 @@ struct ReduceArgs {
     int G;
 };
 
+// Whole iterations in one cooperative launch (nsli_dense.cu).
+struct IterArgs {
+    MapArgs map;               // (part_stat is not used)
+    ReduceArgs red;            // part_dx: two halves of nblk sums (dx^2, y^2)
+    unsigned int *sync;        // grid counters: A, B, C, CTAs that have left
+    unsigned long long *dmax;  // nblk: max |dx_j| of a column block (bits)
+    void *stats;               // 2 x G records (32 bytes each at most)
+    int iters, nblk;
+};
+
 // Grouped launches (continuous batching): per-problem launch parameters and
 // work items.  A problem's items and thread mapping depend only on itself.
 struct GroupProblem {
     MapArgs map;        // rows_base / rows_rem unused; part_y has one row per item
     ReduceArgs red;     // G = number of items of the problem
-    int nt, vpt;        // Map threads owning vectors, vectors per thread
+    int vpt;            // Map vectors per thread
     int red_blocks;     // reduce blocks of this problem
     int first_red;      // index of its first block in the grouped reduce launch
 };
@@ -185,25 +199,26 @@ struct VerifyArgs {
 
 // ---- launchers (nsli_kernels.cu) -------------------------------------------
 constexpr int kMapMaxConsumers = 512;
-constexpr int kMapRowGroup = 8;      // most rows reduced per block barrier
 constexpr int kReduceCols = 32;      // columns per reduce block
-constexpr int kSmemHeader = 2432;    // barriers, flags, warp-sum buffers
-
-// rows per block barrier of the Map kernel for a vectors-per-thread count;
-// a ring slot always holds a multiple of it
-// (eight for one vector per thread with binary32 accumulation: short rows,
-// whose fixed cost per barrier would otherwise dominate; the two halves of
-// the warp-sum buffer hold 1024 bytes each)
-__host__ __device__ constexpr int map_rows_per_group(int vpt, int acc_bytes)
-{
-    return vpt >= 8 ? 1 : (vpt >= 4 ? 2 : (vpt >= 2 || acc_bytes > 4 ? 4 : 8));
-}
+constexpr int kSmemHeader = 2432;    // long-row cluster Map: barriers, flags, warp-sum buffers
+constexpr int kSmemMax = 232448;     // shared memory of a CTA
+constexpr int kLargeTeam = 8;        // teams of this many warps refill the ring through their first warp
+constexpr int kMapMaxStages = 64;    // ring stages of the register-resident Map
+constexpr int kTeamHeader = 12672;    // its barriers, flags, warp sums, statistics and reduce words
 
 int map_vpt_limit(int storage);      // largest vectors-per-thread instance
-// guard: some thread's vectors fall outside the row (nv < threads * vpt)
-cudaError_t map_prepare(int storage, int vpt, bool guard, size_t smem);
-cudaError_t map_launch(int storage, int vpt, bool guard, int grid, int consumers, size_t smem,
-                       cudaStream_t s, const MapArgs &a);
+// the Map of a handle: register-resident rows (vpt > 0) or long rows
+cudaError_t map_launch(int storage, int vpt, int grid, size_t smem, cudaStream_t s, const MapArgs &a);
+cudaError_t long_prepare(int storage, size_t smem);
+// register-resident rows: most rows per group (a ring slot) of the instances
+// for vpt, their shared-memory limit, and the launch
+int team_rg_max(int vpt, bool f64);
+// threads of a block: its teams, and at least eight warps (the barriers' set-up
+// and the reduce of iterate_kernel spread over them)
+int team_threads(int teams, int team_warps);
+cudaError_t team_prepare(int storage, int vpt, int rg, int threads, int *iter_blocks_per_sm);
+cudaError_t iterate_launch(int storage, int vpt, int grid, size_t smem, cudaStream_t s, const IterArgs &a);
+cudaError_t team_launch(int storage, int vpt, int grid, size_t smem, cudaStream_t s, const MapArgs &a);
 // long rows on clusters of C CTAs: set the kernel's shared memory and return
 // how many clusters can be resident at once (0: the shape does not fit)
 cudaError_t cluster_prepare(int storage, int vpt, int rg, int C, size_t smem, int *clusters);
@@ -212,7 +227,7 @@ cudaError_t reduce_only_launch(bool f64, int grid, cudaStream_t s, const ReduceA
                                double *y_out);
 cudaError_t verify_launch(int storage, int grid, cudaStream_t s, const VerifyArgs &a);
 // grouped launches over the problems of a pool (one storage type)
-cudaError_t map_group_prepare(int storage, size_t smem);
+cudaError_t map_group_prepare(int storage);
 cudaError_t map_group_launch(int storage, int items, size_t smem, cudaStream_t s, const GroupProblem *probs,
                              const GroupItem *it);
 cudaError_t reduce_group_launch(bool f64, int blocks, cudaStream_t s, const GroupProblem *probs,
@@ -287,6 +302,7 @@ struct StateBegin {
     long long tick;      // >= 0: set the tick
     double *rtab;        // non-NULL: write lambda / h to rtab[h], h = 0..rtab_m (0 for h = 0)
     long long rtab_m;
+    unsigned int *sync;  // non-NULL: the four grid counters of iterate_kernel, cleared
 };
 cudaError_t state_begin_launch(cudaStream_t s, DevState *st, const StateBegin &b);
 cudaError_t state_resume_launch(cudaStream_t s, DevState *st);
