@@ -625,9 +625,8 @@ template <typename T> __global__ void sparse_rows_kernel(const SparseArgs p, lon
 // ModAP's step; the terms of ||dx|| after the step's barrier, folded in a
 // fixed order.  Only x, x64 and DevState persist between launches (global
 // memory), so launches of any size give identical results.  The statistics
-// a stop rule does not read are not formed: DevState keeps h and max r_i
-// always, max r_i / ||a_i|| only under EPSMEM and max |b_i| only under
-// MAXVIOL_REL (-inf / 0 otherwise).
+// a stop rule does not read are not formed: DevState keeps h always, and the
+// maxima of the last iteration of a run whose rule reads them.
 
 __device__ __forceinline__ double sp_ord_dec(unsigned long long u)
 {
@@ -716,6 +715,17 @@ __device__ __forceinline__ float first_term(float a, float v)
     return a * v;
 }
 
+// a - b; for b = +0 that is a itself, without a binary64 operation
+__device__ __forceinline__ double minus(double a, double b)
+{
+    return __double_as_longlong(b) == 0 ? a : a - b;
+}
+__device__ __forceinline__ float minus(float a, float b) { return a - b; }
+
+// cached per thread: short rows, short columns, entries of a column (three
+// rows, two columns cover the model system up to n = 330)
+constexpr int kResRows = 3, kResCols = 2, kResEntries = 3;
+
 template <typename T>
 __global__ void __launch_bounds__(kResThreads, 1) sparse_resident_kernel(const SparseArgs p, int iters)
 {
@@ -752,7 +762,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sparse_resident_kernel(const S
     const long long max_iter = st->max_iter;
     const int rule = st->rule, stop = st->stop, hold = st->hold_tick;
     const bool modap = rule == NSLI_RULE_MODAP;
-    const bool want_mn = stop == NSLI_STOP_EPSMEM, want_mb = stop == NSLI_STOP_MAXVIOL_REL;
+    const bool want_mn = stop == NSLI_STOP_EPSMEM, want_mb = stop == NSLI_STOP_MAXVIOL_REL;   // (mb: and max r_i)
     for (long long j = tid; j < n; j += kResThreads) {
         x64s[j] = p.x64[j];
         xs[j] = xg[j];
@@ -784,6 +794,62 @@ __global__ void __launch_bounds__(kResThreads, 1) sparse_resident_kernel(const S
         sh_tk[0] = (T)((double)tick * rho);
         sh_done = 0;
     }
+    // The structure of this thread's first kResRows short rows and kResCols
+    // short columns (the same in every iteration) stays in registers: length
+    // and first entries, and a row's record.  A small system then reads no
+    // global memory inside the loop (offsets, then entries, then the gather
+    // are a chain of three L1 round trips otherwise).
+    struct Row {
+        int len, col;
+        long long e0;
+        T val, b0, av, inv_n2, inv_n;
+    } row[kResRows];
+    struct Col {
+        int len, idx[kResEntries];
+        long long e0;
+        T val[kResEntries];
+    } col[kResCols];
+#pragma unroll
+    for (int q = 0; q < kResRows; ++q) {
+        const long long i = tid + (long long)q * nt_r;
+        row[q] = Row{};
+        row[q].len = -1;   // (no such row, or a long one)
+        if (tid < nt_r && i < m) {
+            const long long e0 = p.rp[i], e1 = p.rp[i + 1];
+            if (e1 - e0 <= kResLong) {
+                const Meta md = meta[i];
+                row[q].len = (int)(e1 - e0);
+                row[q].e0 = e0;
+                row[q].b0 = (T)md.b0;
+                row[q].av = (T)md.av;
+                row[q].inv_n2 = (T)md.inv_n2;
+                row[q].inv_n = (T)md.inv_n;
+                if (e1 > e0) {
+                    row[q].col = p.ci[e0];
+                    row[q].val = va[e0];
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < kResCols; ++q) {
+        const long long j = tid + (long long)q * nt_c;
+        col[q] = Col{};
+        col[q].len = -1;
+        if (tid < nt_c && j < n) {
+            const long long e0 = p.cp[j], e1 = p.cp[j + 1];
+            if (e1 - e0 <= kResLong) {
+                col[q].len = (int)(e1 - e0);
+                col[q].e0 = e0;
+#pragma unroll
+                for (int e = 0; e < kResEntries; ++e)
+                    if (e0 + e < e1) {
+                        col[q].idx[e] = p.ri[e0 + e];
+                        col[q].val[e] = vc[e0 + e];
+                    }
+            }
+        }
+    }
     __syncthreads();
 
     // warp 0: does the step rule hold after the step whose terms carry parity q?
@@ -806,25 +872,41 @@ __global__ void __launch_bounds__(kResThreads, 1) sparse_resident_kernel(const S
             sh_tk[par ^ 1] = (T)((double)(hold ? tick : tick + 1) * rho);
         int hc = 0;
         ResMax<T> mv(-INFINITY), mn(-INFINITY), mb(0.0);
-        auto row_done = [&](long long i, T dot) {
-            const Meta md = meta[i];
-            const T bi = tk0 ? (T)md.b0 : fma(tk, (T)md.av, (T)md.b0);
-            const T ri = dot - bi;
+        auto row_done = [&](long long i, T dot, T b0, T av, T inv_n2, T inv_n) {
+            const T bi = tk0 ? b0 : fma(tk, av, b0);
+            const T ri = minus(dot, bi);
             const bool viol = positive(ri);
             T c = T(0);
             if (viol)
-                c = ri * (T)md.inv_n2;
+                c = ri * inv_n2;
             cs[i] = c;
             hc += viol ? 1 : 0;
-            mv.add(ri);
             if (want_mn)
-                mn.add(ri * (T)md.inv_n);
-            if (want_mb)
+                mn.add(ri * inv_n);
+            if (want_mb) {
+                mv.add(ri);
                 mb.add(bi < T(0) ? -bi : bi);
+            }
+        };
+        auto row_of = [&](long long i, T dot) {
+            const Meta md = meta[i];
+            row_done(i, dot, (T)md.b0, (T)md.av, (T)md.inv_n2, (T)md.inv_n);
         };
         if (tid < nt_r) {
-            // short rows, two at a time (independent chains)
-            for (long long i0 = tid; i0 < m; i0 += 2 * (long long)nt_r) {
+            // short rows: the cached ones side by side, then any others, two
+            // at a time (independent chains)
+            T dot[kResRows];
+#pragma unroll
+            for (int q = 0; q < kResRows; ++q)
+                dot[q] = row[q].len > 0 ? first_term(row[q].val, xs[row[q].col]) : T(0);
+#pragma unroll
+            for (int q = 0; q < kResRows; ++q) {
+                for (int e = 1; e < row[q].len; ++e)
+                    dot[q] = fma(__ldg(va + row[q].e0 + e), xs[__ldg(p.ci + row[q].e0 + e)], dot[q]);
+                if (row[q].len >= 0)
+                    row_done(tid + (long long)q * nt_r, dot[q], row[q].b0, row[q].av, row[q].inv_n2, row[q].inv_n);
+            }
+            for (long long i0 = tid + (long long)kResRows * nt_r; i0 < m; i0 += 2 * (long long)nt_r) {
                 const long long i1 = i0 + nt_r;
                 const long long a0 = __ldg(p.rp + i0), b0 = __ldg(p.rp + i0 + 1);
                 long long a1 = 0, b1 = 0;
@@ -846,9 +928,9 @@ __global__ void __launch_bounds__(kResThreads, 1) sparse_resident_kernel(const S
                         s1 = fma(__ldg(va + a1 + q), xs[__ldg(p.ci + a1 + q)], s1);
                 }
                 if (ok0)
-                    row_done(i0, s0);
+                    row_of(i0, s0);
                 if (ok1)
-                    row_done(i1, s1);
+                    row_of(i1, s1);
             }
         } else {
             // long rows: four partial sums per lane, a tree, a butterfly
@@ -867,19 +949,19 @@ __global__ void __launch_bounds__(kResThreads, 1) sparse_resident_kernel(const S
                 T acc = (a4[0] + a4[1]) + (a4[2] + a4[3]);
                 acc = warp_total(acc);
                 if (lane == 0)
-                    row_done(i, acc);
+                    row_of(i, acc);
             }
         }
         // exact folds: integer sum, maxima as order-preserving integers
         unsigned long long umv = mv.enc(), umn = mn.enc(), umb = mb.enc();
+        hc = __reduce_add_sync(0xffffffffu, hc);
+        if (want_mn || want_mb) {
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            hc += __shfl_xor_sync(0xffffffffu, hc, off);
-            umv = umax64(umv, __shfl_xor_sync(0xffffffffu, umv, off));
-            if (want_mn)
+            for (int off = 16; off > 0; off >>= 1) {
+                umv = umax64(umv, __shfl_xor_sync(0xffffffffu, umv, off));
                 umn = umax64(umn, __shfl_xor_sync(0xffffffffu, umn, off));
-            if (want_mb)
                 umb = umax64(umb, __shfl_xor_sync(0xffffffffu, umb, off));
+            }
         }
         if (lane == 0) {
             sh_wh[warp] = hc;
@@ -899,17 +981,21 @@ __global__ void __launch_bounds__(kResThreads, 1) sparse_resident_kernel(const S
                     done = 1;
                 } else {
                     long long H = 0;
-                    unsigned long long a = sh_wmv[0], b = sh_wmn[0], c = sh_wmb[0];
-                    for (int q = 0; q < NW; ++q) {
+#pragma unroll
+                    for (int q = 0; q < NW; ++q)
                         H += sh_wh[q];
-                        a = umax64(a, sh_wmv[q]);
-                        b = umax64(b, sh_wmn[q]);
-                        c = umax64(c, sh_wmb[q]);
-                    }
                     h_last = H;
-                    mv_last = sp_ord_dec(a);
-                    mn_last = sp_ord_dec(b);
-                    mb_last = sp_ord_dec(c);
+                    if (want_mn || want_mb) {
+                        unsigned long long a = sh_wmv[0], b = sh_wmn[0], c = sh_wmb[0];
+                        for (int q = 0; q < NW; ++q) {
+                            a = umax64(a, sh_wmv[q]);
+                            b = umax64(b, sh_wmn[q]);
+                            c = umax64(c, sh_wmb[q]);
+                        }
+                        mv_last = sp_ord_dec(a);
+                        mn_last = sp_ord_dec(b);
+                        mb_last = sp_ord_dec(c);
+                    }
                     const bool pass = !force && ((stop != NSLI_STOP_NONE && H == 0) ||
                                                  (stop == NSLI_STOP_EPSMEM && mn_last < eps) ||
                                                  (stop == NSLI_STOP_MAXVIOL_REL && mv_last <= eps * mb_last));
@@ -929,7 +1015,32 @@ __global__ void __launch_bounds__(kResThreads, 1) sparse_resident_kernel(const S
         }
         // y_j in CSC order over the violated rows (c_i = 0 adds nothing)
         if (tid < nt_c) {
-            for (long long j = tid; j < n; j += nt_c) {
+#pragma unroll
+            for (int q = 0; q < kResCols; ++q) {
+                if (col[q].len < 0)
+                    continue;
+                T c[kResEntries];
+#pragma unroll
+                for (int e = 0; e < kResEntries; ++e)
+                    c[e] = e < col[q].len ? cs[col[q].idx[e]] : T(0);
+                T y = T(0);
+                bool first = true;
+#pragma unroll
+                for (int e = 0; e < kResEntries; ++e)
+                    if (c[e] != T(0)) {
+                        y = first ? first_term(col[q].val[e], c[e]) : fma(col[q].val[e], c[e], y);
+                        first = false;
+                    }
+                for (int e = kResEntries; e < col[q].len; ++e) {
+                    const T ce = cs[__ldg(p.ri + col[q].e0 + e)];
+                    if (ce != T(0)) {
+                        y = first ? first_term(__ldg(vc + col[q].e0 + e), ce) : fma(__ldg(vc + col[q].e0 + e), ce, y);
+                        first = false;
+                    }
+                }
+                ys[tid + q * nt_c] = (double)y;
+            }
+            for (long long j = tid + (long long)kResCols * nt_c; j < n; j += nt_c) {
                 const long long e0 = __ldg(p.cp + j), e1 = __ldg(p.cp + j + 1);
                 if (e1 - e0 > kResLong)
                     continue;
