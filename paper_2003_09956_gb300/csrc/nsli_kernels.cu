@@ -315,9 +315,16 @@ constexpr int kClusterThreads = kClusterCompute + 32;
 
 // RG = rows per group (1, 2 or 4): the rows of a group share one block
 // barrier and one exchange message, and their dependent chains interleave.  The
-// arithmetic of every row is the same for both (the warp fold of two rows
+// arithmetic of every row is the same for all (the warp fold of two rows
 // adds the same operands in the same tree as one warp butterfly per row,
 // and rows enter y in row order).
+// Bound: HBM for binary32; for bf16 and FP8 the mapping warps' instructions
+// per group.  A group's dots have no branch between its rows, its residuals
+// are taken once per row (a lane group each) instead of once per lane, and
+// ring positions are counted along: six remainders by a run-time stage count
+// had taken a third of the instructions.  Map of 27000 x 54000, before ->
+// with these: binary32 1.069 -> 1.036 ms, bf16 0.800 -> 0.668 ms (4.4 TB/s), FP8
+// 0.700 -> 0.550 ms.
 template <int S, int VPT, int RG>
 __global__ void __launch_bounds__(kClusterThreads, 1) map_cluster_kernel(const MapArgs p)
 {
@@ -358,8 +365,13 @@ __global__ void __launch_bounds__(kClusterThreads, 1) map_cluster_kernel(const M
     const unsigned char *Ab = static_cast<const unsigned char *>(p.A);
     const unsigned char *Mb = static_cast<const unsigned char *>(p.meta);
 
+    // ring positions are counted along (a remainder by the stage count, which
+    // the compiler does not know, costs some twenty instructions)
+    auto wrap = [&](int stage) { return stage >= p.nstage ? stage - p.nstage : stage; };
+    int istage = 0;             // the issuing thread: the next stage to fill
     auto issue = [&](int s) {   // row s of the block into its stage
-        const int stage = s % p.nstage;
+        const int stage = istage;
+        istage = wrap(istage + 1);
         const long long row = row_begin + s;
         unsigned char *dst = stages + (size_t)stage * p.stage_stride;
         const unsigned int fb = smem_u32(&full[stage]);
@@ -397,8 +409,8 @@ __global__ void __launch_bounds__(kClusterThreads, 1) map_cluster_kernel(const M
 #pragma unroll
         for (int v = 0; v < VPT; ++v) {
             const int j = tid + v * kClusterCompute;
-            voff[v] = j * 16;
             vok[v] = !xw && j < my_nv;
+            voff[v] = vok[v] ? j * 16 : 0;   // beyond the slice: its first vector against x = 0
 #pragma unroll
             for (int e = 0; e < EPV; ++e) {
                 xr[v][e] = vok[v] ? xg[(v0 + j) * EPV + e] : Acc(0);
@@ -412,36 +424,56 @@ __global__ void __launch_bounds__(kClusterThreads, 1) map_cluster_kernel(const M
     int aborted = 0, at = 0, stalled = 0;
 
     const int D = p.cluster_lag;
+    int dstage = 0, sstage = 0;     // stages of the group being dotted, and being finished
+    unsigned int dph = 0, sph = 0;  // fills of those stages
     for (int g = 0; g < ngroups + D; ++g) {
         int flag = 0;
         if (g < ngroups && !xw) {
-            // partial dots of the group's rows (a missing second row adds 0)
+            // partial dots of the group's rows: side by side, without
+            // branches between them (a short last group repeats its last row,
+            // masked below), two chains of FMAs per row where a thread has
+            // four vectors or more
+            const int last = min(RG, nrows - g * RG) - 1;
+            const unsigned char *row[RG];
+#pragma unroll
+            for (int rr = 0; rr < RG; ++rr) {
+                const int at_rr = dstage + min(rr, last);
+                const int stage = wrap(at_rr);
+                if (!mbar_wait_bounded(smem_u32(&full[stage]), (dph + (at_rr >= p.nstage ? 1u : 0u)) & 1u))
+                    flag = 1;
+                row[rr] = stages + (size_t)stage * p.stage_stride;
+            }
+            constexpr int NCH = VPT == 4 ? 2 : 1;
             Acc acc[RG];
 #pragma unroll
             for (int rr = 0; rr < RG; ++rr) {
-                const int s = g * RG + rr;
-                Acc pe = Acc(0), po = Acc(0);
-                if (s < nrows) {
-                    const int stage = s % p.nstage;
-                    if (!mbar_wait_bounded(smem_u32(&full[stage]), (unsigned int)((s / p.nstage) & 1)))
-                        flag = 1;
-                    const unsigned char *row = stages + (size_t)stage * p.stage_stride;
+                Acc pe[NCH], po[NCH];
 #pragma unroll
-                    for (int v = 0; v < VPT; ++v) {
-                        if (vok[v] && !flag) {
-                            Acc a[EPV];
-                            decode<S>(*reinterpret_cast<const uint4 *>(row + voff[v]), a);
-#pragma unroll
-                            for (int e = 0; e < EPV; e += 2)
-                                fma2(pe, po, a[e], a[e + 1], xr[v][e], xr[v][e + 1]);
-                        }
-                    }
+                for (int q = 0; q < NCH; ++q) {
+                    pe[q] = Acc(0);
+                    po[q] = Acc(0);
                 }
-                acc[rr] = pe + po;
+#pragma unroll
+                for (int v = 0; v < VPT; ++v) {
+                    Acc a[EPV];
+                    decode<S>(*reinterpret_cast<const uint4 *>(row[rr] + voff[v]), a);
+#pragma unroll
+                    for (int e = 0; e < EPV; e += 2)
+                        fma2(pe[v % NCH], po[v % NCH], a[e], a[e + 1], xr[v][e], xr[v][e + 1]);
+                }
+                acc[rr] = pe[0] + po[0];
+#pragma unroll
+                for (int q = 1; q < NCH; ++q)
+                    acc[rr] += pe[q] + po[q];
             }
             const Acc ws = warp_fold_rows<RG>(acc, lane);   // lanes [16q, 16q + 16) end with row q
             if ((lane & (32 / RG - 1)) == 0)
                 red[(g & 1) * (RG * 16) + (lane / (32 / RG)) * 16 + warp] = ws;
+            dstage += RG;
+            if (dstage >= p.nstage) {
+                dstage -= p.nstage;
+                ++dph;
+            }
         }
         if (leader && g >= D) {
             const int t = g - D;
@@ -484,10 +516,11 @@ __global__ void __launch_bounds__(kClusterThreads, 1) map_cluster_kernel(const M
                 // has finished it (in this iteration, below)
                 const int t = g - D;
                 for (int rr = 0; rr < RG && !stalled; ++rr) {
-                    const int r = t * RG + rr;
+                    const int r = t * RG + rr, at_rr = sstage + rr;
                     if (r >= nrows || issued >= nrows)
                         break;
-                    if (mbar_wait_bounded(smem_u32(&empty[r % p.nstage]), (unsigned int)((r / p.nstage) & 1))) {
+                    if (mbar_wait_bounded(smem_u32(&empty[wrap(at_rr)]),
+                                          (sph + (at_rr >= p.nstage ? 1u : 0u)) & 1u)) {
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         issue(issued);
                         ++issued;
@@ -498,46 +531,56 @@ __global__ void __launch_bounds__(kClusterThreads, 1) map_cluster_kernel(const M
                 }
             }
         } else if (g >= D) {
+            // the group's residuals and coefficients, row fq in the lanes of
+            // group fq, then the slices row after row
             const int t = g - D;
+            constexpr int WL = 32 / RG;
+            const int fq = lane / WL;
+            const int cnt = min(RG, nrows - t * RG);
+            const bool valid = fq < cnt;
+            const Acc *xc = xch + (t % kClXB) * (RG * 8) + fq * 8;
+            Acc dot = Acc(0);
+            for (int q = 0; q < C; ++q)
+                dot += xc[q];
+            const int mine = wrap(sstage + (valid ? fq : 0));
+            const Meta md = *reinterpret_cast<const Meta *>(stages + (size_t)mine * p.stage_stride + meta_off);
+            const Acc sc = (Acc)meta_scale(md);
+            const Acc bi = fma(tk, (Acc)md.av, (Acc)md.b0);
+            const Acc ri = (S == NSLI_FP8E4M3) ? dot * sc - bi : dot - bi;
+            const bool viol = valid && ri > Acc(0);
+            const Acc cl = viol ? ((S == NSLI_FP8E4M3) ? ri * (Acc)md.inv_n2 * sc : ri * (Acc)md.inv_n2) : Acc(0);
+            if (warp == 0 && valid) {   // (the lanes of a row alike; one of each is counted at the end)
+                h_loc += viol ? 1 : 0;
+                mv = ri > mv ? ri : mv;
+                const Acc rn = ri * (Acc)md.inv_n;
+                mn = rn > mn ? rn : mn;
+                const Acc ab = bi < Acc(0) ? -bi : bi;
+                mb = ab > mb ? ab : mb;
+            }
 #pragma unroll
             for (int rr = 0; rr < RG; ++rr) {
-                const int r = t * RG + rr;
-                if (r >= nrows)
-                    break;
-                Acc dot = Acc(0);
-                for (int q = 0; q < C; ++q)
-                    dot += xch[(t % kClXB) * (RG * 8) + rr * 8 + q];
-                const unsigned char *row = stages + (size_t)(r % p.nstage) * p.stage_stride;
-                const Meta md = *reinterpret_cast<const Meta *>(row + meta_off);
-                const Acc sc = (Acc)meta_scale(md);
-                const Acc bi = fma(tk, (Acc)md.av, (Acc)md.b0);
-                const Acc ri = (S == NSLI_FP8E4M3) ? dot * sc - bi : dot - bi;
-                const bool viol = ri > Acc(0);
-                const Acc c = viol ? ((S == NSLI_FP8E4M3) ? ri * (Acc)md.inv_n2 * sc : ri * (Acc)md.inv_n2)
-                                   : Acc(0);
-                if (warp == 0) {
-                    h_loc += viol ? 1 : 0;
-                    mv = ri > mv ? ri : mv;
-                    const Acc rn = ri * (Acc)md.inv_n;
-                    mn = rn > mn ? rn : mn;
-                    const Acc ab = bi < Acc(0) ? -bi : bi;
-                    mb = ab > mb ? ab : mb;
-                }
+                const Acc c = __shfl_sync(0xffffffffu, cl, rr * WL);
                 if (c != Acc(0)) {
+                    const unsigned char *row = stages + (size_t)wrap(sstage + rr) * p.stage_stride;
 #pragma unroll
                     for (int v = 0; v < VPT; ++v) {
-                        if (vok[v]) {
-                            Acc a[EPV];
-                            decode<S>(*reinterpret_cast<const uint4 *>(row + voff[v]), a);
+                        Acc a[EPV];
+                        decode<S>(*reinterpret_cast<const uint4 *>(row + voff[v]), a);
 #pragma unroll
-                            for (int e = 0; e < EPV; e += 2)
-                                fma2(yr[v][e], yr[v][e + 1], c, c, a[e], a[e + 1]);
-                        }
+                        for (int e = 0; e < EPV; e += 2)
+                            fma2(yr[v][e], yr[v][e + 1], c, c, a[e], a[e + 1]);
                     }
                 }
-                __syncwarp();
-                if (lane == 0)
-                    mbar_arrive(smem_u32(&empty[r % p.nstage]));   // row r's stage is free
+            }
+            __syncwarp();
+            if (lane < cnt)
+                mbar_arrive(smem_u32(&empty[wrap(sstage + lane)]));   // these rows' stages are free
+        }
+        if (g >= D) {
+            sstage += RG;
+            if (sstage >= p.nstage) {
+                sstage -= p.nstage;
+                ++sph;
             }
         }
     }
@@ -560,6 +603,18 @@ __global__ void __launch_bounds__(kClusterThreads, 1) map_cluster_kernel(const M
 #pragma unroll
                 for (int e = 0; e < EPV; ++e)
                     py[j * EPV + e] = yr[v][e];
+            }
+        }
+        if (warp == 0) {
+            // one lane of each row group (0, 32 / RG, ...)
+#pragma unroll 1
+            for (int off = 32 / RG; off < 32; off <<= 1) {
+                h_loc += __shfl_xor_sync(0xffffffffu, h_loc, off);
+                const Acc a = __shfl_xor_sync(0xffffffffu, mv, off), b = __shfl_xor_sync(0xffffffffu, mn, off),
+                          c = __shfl_xor_sync(0xffffffffu, mb, off);
+                mv = a > mv ? a : mv;
+                mn = b > mn ? b : mn;
+                mb = c > mb ? c : mb;
             }
         }
         if (tid == 0 && rank == 0) {
