@@ -78,6 +78,8 @@ __device__ __forceinline__ bool give_up(unsigned int polls, long long t0)
 // kWaitLimitCycles or when another role has.
 __device__ __forceinline__ bool team_wait(unsigned int bar, unsigned int parity)
 {
+    if (mbar_test(bar, parity))
+        return true;
     const long long t0 = clock64();
     for (unsigned int it = 0; !mbar_test(bar, parity); ++it)
         if (give_up(it, t0))
@@ -211,7 +213,8 @@ __device__ __forceinline__ void ring_issue(const MapArgs &p, const RingSource &s
     bulk_g2s(dst, src.A + r0 * p.row_bytes, bytesA, fb);
     bulk_g2s(dst + (unsigned int)R * (unsigned int)p.row_bytes, src.meta + r0 * 32, bytesM, fb);
     // the fill's barrier phase is open: teams may wait for it (slot_wait)
-    __threadfence_block();
+    if (p.teams > 1)
+        __threadfence_block();
     reinterpret_cast<volatile int *>(smem + kHIssued)[stage] += 1;
 }
 
@@ -239,6 +242,8 @@ __device__ __forceinline__ bool slot_wait(const MapArgs &p, int stage, unsigned 
     const volatile int *issued = reinterpret_cast<const volatile int *>(smem + kHIssued) + stage;
     const unsigned int bar = smem_u32(smem + kHFull) + 8u * stage;
     const bool several = p.teams > 1;
+    if (!several && mbar_test(bar, fill & 1u))
+        return true;
     const long long t0 = clock64();
     for (unsigned int it = 0; (several && (unsigned)*issued <= fill) || !mbar_test(bar, fill & 1u); ++it)
         if (give_up(it, t0))
