@@ -59,7 +59,7 @@ struct nsli_solver {
     PartStat *part_stat = nullptr;
     DevState *st = nullptr;
     VerOut *ver = nullptr;
-    int *flags = nullptr;
+    int *flags = nullptr;         // device address of flags_host
 
     // lambda / h, h = 0..m, for the relaxed step (filled when a run begins
     // with a step size other than the one it holds)
@@ -68,7 +68,9 @@ struct nsli_solver {
 
     DevState *st_host = nullptr;  // pinned
     VerOut *ver_host = nullptr;   // pinned
-    int *flags_host = nullptr;    // pinned
+    // input-check flags, pinned and mapped: kernels write them only when an
+    // input is bad, so a call neither clears nor copies them on the device
+    int *flags_host = nullptr;
 
     // sparse A (nsli_create_csr): CSR + CSC copies, see nsli_sparse.cu
     bool sparse = false;
@@ -144,7 +146,7 @@ void free_all(nsli_solver *h)
     if (h->graph)
         cudaGraphExecDestroy(h->graph);
     void *dev[] = {h->A, h->meta, h->x, h->part_y, h->b0_64, h->av_64, h->n2_64, h->part_dx, h->ybuf, h->shard_dx,
-                   h->dtmp, h->scale, h->part_stat, h->st, h->ver, h->flags,
+                   h->dtmp, h->scale, h->part_stat, h->st, h->ver,
                    (h->x64 != h->x) ? (void *)h->x64 : nullptr,
                    (h->n2_meta != h->n2_64) ? (void *)h->n2_meta : nullptr,
                    h->rp, h->cp, h->ci, h->ri, h->row_cnt, h->col_cnt, h->row_pieces, h->col_pieces, h->iter_sync, h->iter_dmax, h->iter_stats,
@@ -490,11 +492,38 @@ int validate_params(nsli_solver *h, const nsli_params *p)
     return NSLI_OK;
 }
 
+// Every call that checks its inputs clears the flags first (no device work
+// that could raise them is in flight: such calls end with read_flags).
+void clear_flags(nsli_solver *h) { *(volatile int *)h->flags_host = 0; }
+
+cudaError_t alloc_flags(nsli_solver *h)
+{
+    cudaError_t e = cudaHostAlloc((void **)&h->flags_host, sizeof(int), cudaHostAllocMapped);
+    if (e == cudaSuccess)
+        e = cudaHostGetDevicePointer((void **)&h->flags, h->flags_host, 0);
+    if (e == cudaSuccess)
+        clear_flags(h);
+    return e;
+}
+
+// May a kernel of the handle read doubles at p directly?  (memory of its own
+// device, aligned; everything else goes through a staging copy)
+bool readable_by_kernel(const nsli_solver *h, const double *p)
+{
+    cudaPointerAttributes at;
+    if (reinterpret_cast<uintptr_t>(p) % 8 != 0)
+        return false;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == h->device;
+}
+
 int read_flags(nsli_solver *h)
 {
-    CK(cudaMemcpyAsync(h->flags_host, h->flags, sizeof(int), cudaMemcpyDeviceToHost, h->stream), "read flags");
     CK(cudaStreamSynchronize(h->stream), "synchronize");
-    const int f = *h->flags_host;
+    const int f = *(volatile int *)h->flags_host;
     if (f & PREPF_TIMEOUT)
         return set_err(h, NSLI_ERR_TIMEOUT, "a row copy did not arrive within the wait limit");
     if (f & PREPF_NONFINITE)
@@ -694,13 +723,11 @@ int nsli_create(nsli_handle *out, int64_t m, int64_t n, int32_t storage, int32_t
     CKC(cudaMalloc((void **)&h->dtmp, (size_t)std::max<long long>(m, h->ld) * 8), "allocate staging");
     CKC(cudaMalloc((void **)&h->st, sizeof(DevState)), "allocate state");
     CKC(cudaMalloc((void **)&h->ver, sizeof(VerOut)), "allocate check");
-    CKC(cudaMalloc((void **)&h->flags, sizeof(int)), "allocate flags");
+    CKC(alloc_flags(h), "allocate flags");
     CKC(cudaMallocHost((void **)&h->st_host, sizeof(DevState)), "allocate pinned state");
     CKC(cudaMallocHost((void **)&h->ver_host, sizeof(VerOut)), "allocate pinned check");
-    CKC(cudaMallocHost((void **)&h->flags_host, sizeof(int)), "allocate pinned flags");
 
     CKC(cudaMemsetAsync(h->st, 0, sizeof(DevState), s), "clear state");
-    CKC(cudaMemsetAsync(h->flags, 0, sizeof(int), s), "clear flags");
     CKC(cudaMemsetAsync(h->ybuf, 0, (size_t)h->ld * 8, s), "clear y");
     CKC(cudaMemcpyAsync(h->b0_64, b0, (size_t)m * 8, cudaMemcpyDefault, s), "copy b0");
     if (Av)
@@ -1033,10 +1060,9 @@ int nsli_create_csr(nsli_handle *out, int64_t m, int64_t n, int32_t storage, int
     CKC(cudaMalloc((void **)&h->dtmp, (size_t)std::max<long long>(m, n) * 8), "allocate staging");
     CKC(cudaMalloc((void **)&h->st, sizeof(DevState)), "allocate state");
     CKC(cudaMalloc((void **)&h->ver, sizeof(VerOut)), "allocate check");
-    CKC(cudaMalloc((void **)&h->flags, sizeof(int)), "allocate flags");
+    CKC(alloc_flags(h), "allocate flags");
     CKC(cudaMallocHost((void **)&h->st_host, sizeof(DevState)), "allocate pinned state");
     CKC(cudaMallocHost((void **)&h->ver_host, sizeof(VerOut)), "allocate pinned check");
-    CKC(cudaMallocHost((void **)&h->flags_host, sizeof(int)), "allocate pinned flags");
 
     // values in the storage type (binary32: rounded to nearest, ties to even)
     std::vector<float> va32, vc32;
@@ -1106,7 +1132,6 @@ int nsli_create_csr(nsli_handle *out, int64_t m, int64_t n, int32_t storage, int
     }
 
     CKC(cudaMemsetAsync(h->st, 0, sizeof(DevState), s), "clear state");
-    CKC(cudaMemsetAsync(h->flags, 0, sizeof(int), s), "clear flags");
     CKC(cudaMemsetAsync(h->ybuf, 0, (size_t)n * 8, s), "clear y");
     CKC(cudaMemsetAsync(h->coef, 0, (size_t)m * eb, s), "clear coefficients");
     CKC(cudaMemcpyAsync(h->b0_64, b0, (size_t)m * 8, cudaMemcpyDefault, s), "copy b0");
@@ -1166,9 +1191,15 @@ int nsli_update_b(nsli_handle h, const double *b0, int64_t tick)
     if (!h)
         return NSLI_ERR_ARG;
     if (b0) {
-        CK(cudaMemsetAsync(h->flags, 0, sizeof(int), h->stream), "clear flags");
-        CK(cudaMemcpyAsync(h->b0_64, b0, (size_t)h->m * 8, cudaMemcpyDefault, h->stream), "copy b0");
+        clear_flags(h);
         MetaArgs ma;
+        // device memory: the record kernel reads it and keeps the copy
+        ma.b0_src = readable_by_kernel(h, b0) ? b0 : nullptr;
+        if (!ma.b0_src)
+            CK(cudaMemcpyAsync(h->b0_64, b0, (size_t)h->m * 8, cudaMemcpyDefault, h->stream), "copy b0");
+        ma.b0_keep = h->b0_64;
+        ma.st = h->st;
+        ma.tick = tick;
         ma.meta = h->meta;
         ma.b0_64 = h->b0_64;
         ma.av_64 = h->av_64;
@@ -1178,13 +1209,12 @@ int nsli_update_b(nsli_handle h, const double *b0, int64_t tick)
         ma.flags = h->flags;
         CK(meta_b0_launch(h->storage == NSLI_F64, h->stream, ma), "update row records");
         h->launches += 1;
+        return read_flags(h);
     }
     if (tick >= 0) {
-        const long long t = tick;  // pageable source: staged before the call returns
-        CK(cudaMemcpyAsync(&h->st->tick, &t, sizeof t, cudaMemcpyHostToDevice, h->stream), "set tick");
+        CK(set_tick_launch(h->stream, h->st, tick), "set tick");
+        h->launches += 1;
     }
-    if (b0)
-        return read_flags(h);
     return NSLI_OK;
 }
 
@@ -1205,7 +1235,7 @@ int nsli_update_rows(nsli_handle h, int64_t row0, int64_t rows, int32_t a_dtype,
     if (rows == 0)
         return NSLI_OK;
     cudaStream_t s = h->stream;
-    CK(cudaMemsetAsync(h->flags, 0, sizeof(int), s), "clear flags");
+    clear_flags(h);
     const size_t src_eb = a_dtype == NSLI_F64 ? 8 : 4;
     const bool on_device = is_device_ptr(A);
     // rows per launch: all of them for a device source, else a staged chunk
@@ -1526,9 +1556,11 @@ int nsli_set_x(nsli_handle h, const double *x)
     Trace trace_("nsli_set_x");
     if (!h || !x)
         return NSLI_ERR_ARG;
-    CK(cudaMemsetAsync(h->flags, 0, sizeof(int), h->stream), "clear flags");
-    CK(cudaMemcpyAsync(h->dtmp, x, (size_t)h->n * 8, cudaMemcpyDefault, h->stream), "copy x");
-    CK(x_from_f64_launch(h->storage == NSLI_F64, h->stream, h->dtmp, h->x64, h->x, h->n, h->ld, h->flags),
+    clear_flags(h);
+    const bool direct = readable_by_kernel(h, x);
+    if (!direct)
+        CK(cudaMemcpyAsync(h->dtmp, x, (size_t)h->n * 8, cudaMemcpyDefault, h->stream), "copy x");
+    CK(x_from_f64_launch(h->storage == NSLI_F64, h->stream, direct ? x : h->dtmp, h->x64, h->x, h->n, h->ld, h->flags),
        "convert x");
     h->launches += 1;
     return read_flags(h);

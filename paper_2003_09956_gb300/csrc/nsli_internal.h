@@ -283,6 +283,12 @@ struct MetaArgs {
     long long m;            // rows [row0, row0 + m)
     int *flags;
     long long row0 = 0;
+    // a new right-hand side (meta_b0_launch): from here (device memory), kept
+    // in b0_keep; NULL: from b0_64.  tick >= 0 sets st->tick.
+    const double *b0_src = nullptr;
+    double *b0_keep = nullptr;
+    DevState *st = nullptr;
+    long long tick = -1;
 };
 cudaError_t meta_launch(bool f64, cudaStream_t s, const MetaArgs &a);
 // only the records' b0 (a new right-hand side)
@@ -306,6 +312,7 @@ struct StateBegin {
 };
 cudaError_t state_begin_launch(cudaStream_t s, DevState *st, const StateBegin &b);
 cudaError_t state_resume_launch(cudaStream_t s, DevState *st);
+cudaError_t set_tick_launch(cudaStream_t s, DevState *st, long long tick);
 // sts[i]->tick = ticks[i] and ticks held (device arrays of count entries)
 cudaError_t set_ticks_launch(cudaStream_t s, DevState *const *sts, const long long *ticks, int count);
 cudaError_t stored_rows_launch(int storage, cudaStream_t s, const void *A, const float *scale, long long ld,

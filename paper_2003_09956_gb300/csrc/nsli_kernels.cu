@@ -966,10 +966,18 @@ __global__ void __launch_bounds__(256) meta_kernel(const MetaArgs p)
 template <bool F64> __global__ void __launch_bounds__(256) meta_b0_kernel(const MetaArgs p)
 {
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k == 0 && p.tick >= 0)
+        p.st->tick = p.tick;
     if (k >= p.m)
         return;
     const long long i = p.row0 + k;
-    const double b0 = p.b0_64[i];
+    double b0;
+    if (p.b0_src) {
+        b0 = p.b0_src[k];
+        p.b0_keep[i] = b0;
+    } else {
+        b0 = p.b0_64[i];
+    }
     if (!isfinite(b0))
         atomicOr(p.flags, PREPF_NONFINITE);
     if (F64)
@@ -1041,6 +1049,8 @@ __global__ void set_ticks_kernel(DevState *const *sts, const long long *ticks, i
         sts[i]->hold_tick = 1;
     }
 }
+
+__global__ void set_tick_kernel(DevState *st, long long tick) { st->tick = tick; }
 
 __global__ void state_resume_kernel(DevState *st)
 {
@@ -1267,6 +1277,12 @@ cudaError_t state_begin_launch(cudaStream_t s, DevState *st, const StateBegin &b
 cudaError_t set_ticks_launch(cudaStream_t s, DevState *const *sts, const long long *ticks, int count)
 {
     set_ticks_kernel<<<(count + 127) / 128, 128, 0, s>>>(sts, ticks, count);
+    return cudaGetLastError();
+}
+
+cudaError_t set_tick_launch(cudaStream_t s, DevState *st, long long tick)
+{
+    set_tick_kernel<<<1, 1, 0, s>>>(st, tick);
     return cudaGetLastError();
 }
 
