@@ -224,6 +224,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     unsigned long long *bars = reinterpret_cast<unsigned long long *>(sbase + NSTAGE * kStageBytes);
     unsigned int *tmem_holder = reinterpret_cast<unsigned int *>(bars + kBarCount);
     volatile int *abort = reinterpret_cast<volatile int *>(bars + kBarCount + 1);
+    __shared__ float tks[64];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int BN = e.BN;
@@ -344,7 +345,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         unsigned int aph = 0;
         const long long k = e.st->k;
         const int cur = (int)(k & 1);
-        const float rho = (float)e.st->rho;
+        // the problems' tick terms, once per launch (per row and problem they
+        // were three binary64 operations in the epilogue)
+        const int et = (int)threadIdx.x - 64;
+        if (e.mode == 0 && et < 64)
+            tks[et] = et < e.nprob ? (float)((double)(e.s_off[et] + k) * (double)(float)e.st->rho) : 0.f;
+        asm volatile("bar.sync 2, 128;" ::: "memory");
         for (int w = blockIdx.x; w < e.nwork; w += gridDim.x) {
             const int tile = w % e.mtiles, ks = w / e.mtiles;
             if (!wait_bar(smem_u32(&bars[kBarTFull + acc]), aph, abort))
@@ -370,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     for (int q = 0; q < 16; ++q) {
                         const int p = pc + q;
                         const bool live = p < e.nprob;
-                        const float tk = live ? (float)((double)(e.s_off[p] + k) * (double)rho) : 0.f;
+                        const float tk = tks[p];
                         const float bi = fmaf(tk, av, b0);
                         const float r = (v0[q] + v1[q]) + v2[q] - bi;
                         const bool viol = valid && live && r > 0.f;
@@ -437,27 +443,32 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // y_p[j] = sum over K splits (in order) of the partials; then either the
 // relaxed step of problem p (mode 1) or y written out (mode 2).
-__global__ void finish_kernel(const float *Ypart, int splits, int Pp, int nprob, long long n, long long ldx,
+__global__ void finish_kernel(const float *Ypart, int splits, int Pp, long long n, long long ldx,
                               const int *cnt, const State *st, double *X64, __nv_bfloat16 *Xs, double *Yout,
                               int mode)
 {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long long)nprob * ldx)
-        return;
-    const long long p = t / ldx, j = t % ldx;
+    // one problem per block row: its lambda / h is one binary64 division per
+    // block, not one per thread (some 20 binary64 operations, which bound the
+    // kernel: 18 -> 8 us at 64 problems of n = 8192)
+    const long long p = blockIdx.y, j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ double s_sh;
+    if (mode != 2 && threadIdx.x == 0) {
+        const int hc = cnt[(int)(st->k & 1) * Pp + p];
+        s_sh = hc > 0 ? st->lambda / (double)hc : 0.0;
+    }
+    double y = 0.0;
+    if (j < n)
+        for (int ks = 0; ks < splits; ++ks)
+            y += (double)Ypart[((long long)ks * Pp + p) * ldx + j];
+    __syncthreads();
     if (j >= n)
         return;
-    double y = 0.0;
-    for (int ks = 0; ks < splits; ++ks)
-        y += (double)Ypart[((long long)ks * Pp + p) * ldx + j];
     const long long ix = p * ldx + j;
     if (mode == 2) {
         Yout[ix] = y;
         return;
     }
-    const int cur = (int)(st->k & 1);
-    const int hc = cnt[cur * Pp + p];
-    const double s = hc > 0 ? st->lambda / (double)hc : 0.0;
+    const double s = s_sh;
     const double xn = X64[ix] - s * y;
     X64[ix] = xn;
     __nv_bfloat16 h, m, l;
@@ -696,9 +707,8 @@ cudaError_t launch_gemm(nsli_batch h, int mode)
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess)
         return err;
-    const long long tot = (long long)h->nprob * h->ldn;
-    finish_kernel<<<(unsigned int)((tot + 255) / 256), 256, 0, h->stream>>>(
-        h->Ypart, h->splits, h->Pp, h->nprob, h->n, h->ldn, h->cnt, h->st, h->X64, h->Xs, h->Y, mode);
+    finish_kernel<<<dim3((unsigned int)((h->n + 255) / 256), (unsigned int)h->nprob), 256, 0, h->stream>>>(
+        h->Ypart, h->splits, h->Pp, h->n, h->ldn, h->cnt, h->st, h->X64, h->Xs, h->Y, mode);
     return cudaGetLastError();
 }
 
