@@ -865,26 +865,20 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepArgs p)
 
     // ||a_i||^2 of the stored values: binary64 for binary64 storage, else the
     // double-float accumulation of nsli_sumsq.cuh, folded into binary64 every
-    // 8 entries (fast = 0: the binary64 norms) or not at all (fast = 1: the
-    // norm behind the row records, as in the row-update kernel), and the
-    // block total of sumsq_block_total
+    // 8 entries (fast = 0: the binary64 norms) or the quick two-pair form
+    // (fast = 1: the norm behind the row records, as in the row-update
+    // kernel), and the block total
     double n2 = 0.0;
     SumSq sq = sumsq_init();
-    for (long long j = threadIdx.x; j < p.ld; j += blockDim.x) {
+    QuickSum<S != NSLI_FP8E4M3> quick;
+    auto put = [&](long long j) -> float {   // stores entry j, returns its stored value (0 past n)
         const bool in = j < p.n;
-        if (S == NSLI_F64) {
-            const double v = in ? (p.src_f64 ? s64[j] : (double)s32[j]) : 0.0;
-            if (in && !isfinite(v))
-                bad = 1;
-            static_cast<double *>(p.A)[gi * p.ld + j] = v;
-            n2 += v * v;
-        } else if (S == NSLI_F32) {
+        if (S == NSLI_F32) {
             const float v = in ? (p.src_f64 ? __double2float_rn(s64[j]) : s32[j]) : 0.0f;
             if (in && !(p.src_f64 ? isfinite(s64[j]) : isfinite(v)))
                 bad = 1;
             static_cast<float *>(p.A)[gi * p.ld + j] = v;
-            if (in && isfinite(v))
-                p.fast ? sumsq_add<0>(sq, v) : sumsq_add<8>(sq, v);
+            return v;
         } else if (S == NSLI_BF16) {
             const float a = in ? s32[j] : 0.0f;
             if (in && !isfinite(a))
@@ -893,18 +887,33 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepArgs p)
             // the row invalid, as in the row-update kernel)
             const __nv_bfloat16 q = __float2bfloat16_rn(a);
             static_cast<__nv_bfloat16 *>(p.A)[gi * p.ld + j] = q;
-            const float v = __bfloat162float(q);
-            if (in)
-                p.fast ? sumsq_add<0>(sq, v) : sumsq_add<8>(sq, v);
+            return __bfloat162float(q);
         } else {
             const float a = in ? s32[j] : 0.0f;
             const __nv_fp8_storage_t q = __nv_cvt_float_to_fp8(a * inv_scale, __NV_SATFINITE, __NV_E4M3);
             static_cast<unsigned char *>(p.A)[gi * p.ld + j] = (unsigned char)q;
             const __half_raw hr = __nv_cvt_fp8_to_halfraw(q, __NV_E4M3);
-            const float v = __fmul_rn(__half2float(__half(hr)), scale);   // exact: scale is a power of two
-            if (in)
-                p.fast ? sumsq_add<0>(sq, v) : sumsq_add<8>(sq, v);
+            return __fmul_rn(__half2float(__half(hr)), scale);   // exact: scale is a power of two
         }
+    };
+    if constexpr (S == NSLI_F64) {
+        for (long long j = threadIdx.x; j < p.ld; j += blockDim.x) {
+            const bool in = j < p.n;
+            const double v = in ? (p.src_f64 ? s64[j] : (double)s32[j]) : 0.0;
+            if (in && !isfinite(v))
+                bad = 1;
+            static_cast<double *>(p.A)[gi * p.ld + j] = v;
+            n2 += v * v;
+        }
+    } else if (p.fast) {
+        for (long long j = threadIdx.x; j < p.ld; j += 2 * (long long)blockDim.x) {
+            const float v0 = put(j);
+            const float v1 = j + blockDim.x < p.ld ? put(j + blockDim.x) : 0.0f;
+            quick.add(v0, v1);
+        }
+    } else {
+        for (long long j = threadIdx.x; j < p.ld; j += blockDim.x)
+            sumsq_add<8>(sq, put(j));
     }
     if (bad)
         sbad = 1;
@@ -912,7 +921,17 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepArgs p)
     if constexpr (S != NSLI_F64) {
         __shared__ float2 spair[8];
         __shared__ double sacc[8];
-        t = sumsq_block_total<8>(sq, spair, sacc);   // (synchronises the block)
+        if (p.fast) {
+            t = sumsq_block_total<8>(quick, spair, sacc);   // (synchronises the block)
+        } else {
+            double v = warp_sum(sumsq_value(sq));
+            if (lane == 0)
+                sacc[wid] = v;
+            __syncthreads();
+            if (threadIdx.x == 0)
+                for (int q = 0; q < 8; ++q)
+                    t += sacc[q];
+        }
     } else {
         n2 = warp_sum(n2);
         if (lane == 0)

@@ -12,9 +12,11 @@
 // additions for 8 entries instead of 16 operations).  The pair carries about
 // 48 significant bits, so each group of 8 is summed to within a few units of
 // 2^-48 relative and the result agrees with a binary64 sum to about 1e-14.
-// Without the periodic fold (FOLD = 0) the pair carries the whole per-thread
-// sum: no binary64 work per entry, and sumsq_block_total adds the pairs of a
-// block as double-floats and converts the row total once.
+// The quick norm (SumSq2) has no periodic fold: each thread keeps two such
+// pairs, for its even and its odd entries, side by side in packed binary32x2
+// instructions (13 for two entries instead of 26: the row updates are bound by
+// their instructions), and sumsq_block_total adds the pairs of a block as
+// double-floats and converts the row total once.
 // Values whose square could leave the binary32 normal range (|v| outside
 // [2^-60, 2^60]) are squared and added in binary64 directly.  The order is
 // fixed per thread, so the set-up kernel and the row-update kernel, which
@@ -51,10 +53,10 @@ __device__ __forceinline__ void sumsq_flush(SumSq &q)
     q.k = 0;
 }
 
-// FOLD = 8: fold into binary64 every 8 entries (accurate to ~1e-14: the
-// binary64 norms); FOLD = 0: never until the end (no binary64 work per
-// entry; accurate to ~1e-12 for a few hundred entries per thread, which is
-// ample for the binary32 row records).
+// One entry.  FOLD = 8: folded into binary64 every 8 entries (accurate to
+// ~1e-14: the binary64 norms); FOLD = 0: never (the quick norm of FP8 rows,
+// whose conversions leave no room for the packed form's moves: 1.09 ms per
+// 32768 x 16384 rows updated against 1.13 ms).
 template <int FOLD = 8> __device__ __forceinline__ void sumsq_add(SumSq &q, float v)
 {
     const float a = fabsf(v);
@@ -83,6 +85,89 @@ __device__ __forceinline__ double sumsq_value(SumSq &q)
     return q.acc;
 }
 
+// Packed binary32x2 arithmetic, each half rounded to nearest as the scalar
+// instruction rounds it.
+__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi)
+{
+    return ((unsigned long long)__float_as_uint(hi) << 32) | __float_as_uint(lo);
+}
+__device__ __forceinline__ float f2_lo(unsigned long long v) { return __uint_as_float((unsigned int)v); }
+__device__ __forceinline__ float f2_hi(unsigned long long v) { return __uint_as_float((unsigned int)(v >> 32)); }
+__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+// a - b (the product with -1 is exact, so the sum is rounded once)
+__device__ __forceinline__ unsigned long long f2_sub(unsigned long long a, unsigned long long b)
+{
+    return f2_fma(b, 0xbf800000bf800000ull, a);
+}
+__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// Two running double-float sums, of a thread's even and odd entries.
+struct SumSq2 {
+    double acc;              // squares outside the binary32 range
+    unsigned long long s, c;
+};
+__device__ __forceinline__ SumSq2 sumsq2_init() { return SumSq2{0.0, 0ull, 0ull}; }
+
+// The next two entries (0 for one that does not exist: a zero changes
+// neither pair, since s is the rounding of s + c).
+__device__ __forceinline__ void sumsq2_add(SumSq2 &q, float v0, float v1)
+{
+    // |v| outside [2^-60, 2^60] and not 0: in binary64
+    const unsigned int u0 = __float_as_uint(v0) & 0x7fffffffu, u1 = __float_as_uint(v1) & 0x7fffffffu;
+    const bool out0 = u0 - 0x21800000u > 0x3c000000u && u0 != 0u, out1 = u1 - 0x21800000u > 0x3c000000u && u1 != 0u;
+    if (out0 || out1) {
+        if (out0) {
+            q.acc = __fma_rn((double)v0, (double)v0, q.acc);
+            v0 = 0.0f;
+        }
+        if (out1) {
+            q.acc = __fma_rn((double)v1, (double)v1, q.acc);
+            v1 = 0.0f;
+        }
+    }
+    const unsigned long long v = f2_pack(v0, v1);
+    const unsigned long long p = f2_mul(v, v);
+    const unsigned long long e = f2_fma(v, v, p ^ 0x8000000080000000ull);
+    const unsigned long long t = f2_add(q.s, p);
+    const unsigned long long bp = f2_sub(t, q.s);
+    const unsigned long long err = f2_add(f2_sub(q.s, f2_sub(t, bp)), f2_sub(p, bp));
+    const unsigned long long c = f2_add(q.c, f2_add(err, e));
+    const unsigned long long s2 = f2_add(t, c);
+    q.c = f2_sub(c, f2_sub(s2, t));
+    q.s = s2;
+}
+
+// The quick norm's accumulator by storage type: the next two entries.
+template <bool PACKED> struct QuickSum;
+template <> struct QuickSum<true> {
+    SumSq2 q = sumsq2_init();
+    __device__ __forceinline__ void add(float v0, float v1) { sumsq2_add(q, v0, v1); }
+};
+template <> struct QuickSum<false> {
+    SumSq q = sumsq_init();
+    __device__ __forceinline__ void add(float v0, float v1)
+    {
+        sumsq_add<0>(q, v0);
+        sumsq_add<0>(q, v1);
+    }
+};
+
 // (s, c) += (s2, c2) for two double-float pairs of non-negative sums:
 // two-sum of the heads (its error is exact, so the result does not depend
 // on the order of the operands), the tails and that error added, and a
@@ -98,30 +183,45 @@ __device__ __forceinline__ void sumsq_pair_add(float &s, float &c, float s2, flo
     s = s3;
 }
 
-// The block total of the per-thread sums of squares taken without the
-// periodic fold (FOLD = 0), for blocks of NW warps: the pairs are added as
-// double-floats in an xor tree within each warp and then in warp order by
+// The block total of the per-thread quick sums, for blocks of NW warps: a
+// thread's two pairs are added, then the threads' as double-floats in an xor
+// tree within each warp and then in warp order by
 // thread 0, and converted to binary64 once; the binary64 parts (squares
 // outside the binary32 range) are added in binary64 only when some thread
 // has one.  Binary32 work instead of a binary64 tree: GB300's binary64 pipe
 // takes a whole warp instruction for each binary64 operation.  Every thread
 // of the block calls it; the result is valid in thread 0.  spair and sacc
 // are shared arrays of NW entries.
-template <int NW>
-__device__ __forceinline__ double sumsq_block_total(const SumSq &q, float2 *spair, double *sacc)
+__device__ __forceinline__ void quick_pair(const QuickSum<true> &a, float &s, float &c, double &acc)
+{
+    s = f2_lo(a.q.s);
+    c = f2_lo(a.q.c);
+    sumsq_pair_add(s, c, f2_hi(a.q.s), f2_hi(a.q.c));
+    acc = a.q.acc;
+}
+__device__ __forceinline__ void quick_pair(const QuickSum<false> &a, float &s, float &c, double &acc)
+{
+    s = a.q.s;
+    c = a.q.c;
+    acc = a.q.acc;
+}
+template <int NW, bool PACKED>
+__device__ __forceinline__ double sumsq_block_total(const QuickSum<PACKED> &q, float2 *spair, double *sacc)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    float s = q.s, c = q.c;
+    float s, c;
+    double acc_in;
+    quick_pair(q, s, c, acc_in);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         const float s2 = __shfl_xor_sync(0xffffffffu, s, off);
         const float c2 = __shfl_xor_sync(0xffffffffu, c, off);
         sumsq_pair_add(s, c, s2, c2);
     }
-    const bool wide = __syncthreads_or(q.acc != 0.0) != 0;   // block-uniform
+    const bool wide = __syncthreads_or(acc_in != 0.0) != 0;   // block-uniform
     double acc = 0.0;
     if (wide) {
-        acc = q.acc;
+        acc = acc_in;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1)
             acc += __shfl_xor_sync(0xffffffffu, acc, off);

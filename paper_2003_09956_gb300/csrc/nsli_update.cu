@@ -251,11 +251,11 @@ template <int S, typename I, bool VEC> __device__ __forceinline__ void update_ro
     }
 
     // pass 1: norm of the stored values (same order and arithmetic as the
-    // set-up kernel's quick norm: thread t adds j = t, t + 256, ... in turn;
-    // binary64 for binary64 storage, else the double-float sum of
-    // nsli_sumsq.cuh folded only at the end); kUnroll loads in flight
+    // set-up kernel's quick norm: thread t adds j = t, t + 256, ... in turn,
+    // two at a time; binary64 for binary64 storage, else the double-float
+    // pairs of nsli_sumsq.cuh); kUnroll loads in flight
     double n2 = 0.0;
-    SumSq sq = sumsq_init();
+    QuickSum<S != NSLI_FP8E4M3> quick;
     for (I j0 = threadIdx.x; j0 < n; j0 += (I)kThreads * kUnroll) {
         if constexpr (S == NSLI_F64) {
             double v[kUnroll];
@@ -277,8 +277,8 @@ template <int S, typename I, bool VEC> __device__ __forceinline__ void update_ro
             // (a row with a non-finite value is rejected below, so its sum
             // may take the value as it is)
 #pragma unroll
-            for (int u = 0; u < kUnroll; ++u)
-                sumsq_add<0>(sq, v[u]);
+            for (int u = 0; u < kUnroll; u += 2)
+                quick.add(v[u], v[u + 1]);
         }
     }
     if (bad)
@@ -290,7 +290,7 @@ template <int S, typename I, bool VEC> __device__ __forceinline__ void update_ro
     if constexpr (S != NSLI_F64) {
         __shared__ float2 spair[kThreads / 32];
         __shared__ double sacc[kThreads / 32];
-        t = sumsq_block_total<kThreads / 32>(sq, spair, sacc);   // (synchronises the block)
+        t = sumsq_block_total<kThreads / 32>(quick, spair, sacc);   // (synchronises the block)
     } else {
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1)
