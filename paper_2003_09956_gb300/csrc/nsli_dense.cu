@@ -134,18 +134,36 @@ template <typename Acc> struct alignas(4 * sizeof(Acc)) RowStat {
         mn = up(mn, o.mn);
         mb = up(mb, o.mb);
     }
-    // over the warp (exact; rolled: see the note on code size)
+    // over the warp, in every lane: integer reductions of one instruction
+    // instead of five shuffles and maxima each (exact; no value is a NaN: up()
+    // never takes one.  A lane's count is at most the rows of the warps or
+    // CTAs it joined; where it could pass 2^26 the 32 lanes' sum is taken as
+    // 64 bits)
     __device__ __forceinline__ void fold()
     {
-#pragma unroll 1
-        for (int off = 16; off > 0; off >>= 1) {
-            RowStat o;
-            o.h = __shfl_xor_sync(0xffffffffu, h, off);
-            o.mv = __shfl_xor_sync(0xffffffffu, mv, off);
-            o.mn = __shfl_xor_sync(0xffffffffu, mn, off);
-            o.mb = __shfl_xor_sync(0xffffffffu, mb, off);
-            join(o);
+        if constexpr (sizeof(Acc) == 8) {
+            const unsigned int lo = (unsigned int)(h & 0x3ffffff), hi = (unsigned int)(h >> 26);
+            h = ((long long)__reduce_add_sync(0xffffffffu, hi) << 26) + __reduce_add_sync(0xffffffffu, lo);
+        } else {
+            h = __reduce_add_sync(0xffffffffu, h);
         }
+        mv = top(mv);
+        mn = top(mn);
+        mb = top(mb);
+    }
+    static __device__ __forceinline__ float top(float v)
+    {
+        // binary32 values order like their bits as signed integers, the
+        // negative ones reversed
+        const int b = __float_as_int(v), k = __reduce_max_sync(0xffffffffu, b < 0 ? b ^ 0x7fffffff : b);
+        return __int_as_float(k < 0 ? k ^ 0x7fffffff : k);
+    }
+    static __device__ __forceinline__ unsigned long long top(unsigned long long v)
+    {
+        const unsigned int hi = __reduce_max_sync(0xffffffffu, (unsigned int)(v >> 32));
+        const unsigned int lo =
+            __reduce_max_sync(0xffffffffu, (unsigned int)(v >> 32) == hi ? (unsigned int)v : 0u);
+        return ((unsigned long long)hi << 32) | lo;
     }
     __device__ __forceinline__ PartStat record() const
     {
@@ -305,7 +323,7 @@ __device__ __forceinline__ bool team_rows(const MapArgs &p, const TeamThread<S, 
     constexpr int EPV = Tr::EPV;
     constexpr int WL = 32 / RG;   // lanes per row in the folded reductions
     // independent chains per row (binary64: one per vector and half, a tree
-    // after it: a dependent binary64 operation costs about 435 cycles)
+    // after it: a dependent binary64 operation costs about 300 cycles)
     constexpr int NCH = sizeof(Acc) == 8 ? V : ((V >= 4 && RG <= 2) ? 2 : 1);
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int R = RG;   // a slot is one row group
@@ -575,7 +593,7 @@ __device__ __forceinline__ void team_finish(const MapArgs &p, const TeamThread<S
             }
     }
     bar_threads(1, nbar);   // (also orders the team statistics)
-    if (threadIdx.x < 32) {
+    if (threadIdx.x < 32 && nt > 1) {   // (one team: warp 0 has them already)
         stat.clear();
         if ((int)threadIdx.x < nt)
             stat = ts[threadIdx.x];
@@ -667,8 +685,8 @@ template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsume
 // What bounds it: large systems, HBM; small ones, the latencies of an
 // iteration's serial steps (x in, rows, y out, A, group sums, step, B: about 8
 // us where the rows take 1 us).  Measured per iteration, separate launches ->
-// here: 2000 x 500 binary32 16.8 -> 8.2 us, 513 x 256 binary64 19.4 -> 11.0 us,
-// 8192 x 2048 binary32 31.0 -> 15.1 us, 20011 x 4099 bf16 82 -> 44 us (ModAP 93
+// here: 2000 x 500 binary32 16.8 -> 8.2 us, 513 x 256 binary64 19.4 -> 8.7 us,
+// 8192 x 2048 binary32 31.0 -> 14.8 us, 20011 x 4099 bf16 82 -> 44 us (ModAP 93
 // -> 48 us), 32768 x 8192 bf16 116 -> 94 us, 131072 x 16384 binary32 1174 ->
 // 1159 us (the left figures with the one-team Map that the teams replace).
 // A: every CTA has written its partial sums and record.  C (ModAP): the
@@ -772,7 +790,7 @@ template <typename Acc> __device__ __forceinline__ RowStat<Acc> stats_of(const R
 {
     RowStat<Acc> s;
     s.clear();
-    constexpr int U = sizeof(Acc) == 8 ? 1 : 5;   // (152 records: one round trip)
+    constexpr int U = sizeof(Acc) == 8 ? 1 : 5;   // (152 records: one round trip; binary64: 2218 us against 2253 at five)
 #pragma unroll 1
     for (int g0 = lane; g0 < G; g0 += 32 * U) {
         RowStat<Acc> q[U];
@@ -806,7 +824,7 @@ template <typename Acc> __device__ __forceinline__ double total_of(const Acc (&v
 // Group grp of NGRP's sum over the partial rows g = grp, grp + NGRP, ... of
 // column j, in that order in the accumulation type (binary64 is slow on this
 // part); binary64: four running sums (g = grp + NGRP (4c + u)) and a tree, a
-// dependent binary64 add costing about 435 cycles.  20 loads are in flight at
+// dependent binary64 add costing about 300 cycles.  20 loads are in flight at
 // a time (all of a group's 19 at 152 partial rows and 8 groups): the sum
 // waits for one round trip to L2, not for three.
 template <typename Acc, int NGRP>
@@ -1411,7 +1429,7 @@ cudaError_t set_smem(const void *fn)
 
 }  // namespace
 
-int team_threads(int teams, int team_warps) { return std::max(256, teams * team_warps * 32); }
+int team_threads(int teams, int team_warps) { return std::max(288, teams * team_warps * 32); }
 
 int team_rg_max(int vpt, bool f64) { return kRgMax(vpt, f64 ? 8 : 4); }
 

@@ -213,8 +213,9 @@ cudaError_t long_prepare(int storage, size_t smem);
 // register-resident rows: most rows per group (a ring slot) of the instances
 // for vpt, their shared-memory limit, and the launch
 int team_rg_max(int vpt, bool f64);
-// threads of a block: its teams, and at least eight warps (the barriers' set-up
-// and the reduce of iterate_kernel spread over them)
+// threads of a block: its teams, and at least nine warps (the set-up of the
+// barriers, and in iterate_kernel eight for a column block's group sums beside
+// the one that takes the counts and maxima)
 int team_threads(int teams, int team_warps);
 cudaError_t team_prepare(int storage, int vpt, int rg, int threads, int *iter_blocks_per_sm);
 cudaError_t iterate_launch(int storage, int vpt, int grid, size_t smem, cudaStream_t s, const IterArgs &a);
