@@ -217,6 +217,7 @@ int team_rg_max(int vpt, bool f64);
 // barriers, and in iterate_kernel eight for a column block's group sums beside
 // the one that takes the counts and maxima)
 int team_threads(int teams, int team_warps);
+cudaError_t team_map_prepare(int storage, int vpt, int rg);
 cudaError_t team_prepare(int storage, int vpt, int rg, int threads, int *iter_blocks_per_sm);
 cudaError_t iterate_launch(int storage, int vpt, int grid, size_t smem, cudaStream_t s, const IterArgs &a);
 cudaError_t team_launch(int storage, int vpt, int grid, size_t smem, cudaStream_t s, const MapArgs &a);

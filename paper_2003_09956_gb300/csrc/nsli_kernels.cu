@@ -8,18 +8,39 @@
 //                  (Section 5 tick, never materialised), and while the row is
 //                  still on chip adds the positive slice (Eq. 7)
 //                  r_i / ||a_i||^2 * a_i into register-resident partial sums
-//                  (rows up to the register-resident limit: nsli_dense.cu;
-//                  longer rows: here).
+//                  (rows up to the register-resident limit: nsli_team.cuh;
+//                  longer rows: below).
 //   reduce_update  deterministic fixed-order sum of the per-CTA partials,
 //                  the stopping test (Eq. 10 and the step rule), and the step
 //                  x <- x - lambda y / h (Eq. 8) or x <- x - lambda y / ||y||
 //                  (Eq. 12), with ||dx|| in binary64.
 // Plus the set-up kernels (quantisation of A, binary64 row norms, per-row
 // records) and the binary64 feasibility check (Eq. 10 on the stored A).
-#include "nsli_map.cuh"
+#include "nsli_team.cuh"
 #include "nsli_sumsq.cuh"
 
 namespace nsli {
+
+namespace {
+
+// One problem: CTA b maps its contiguous balanced block of rows.
+template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsumers, 1) map_kernel(const MapArgs p)
+{
+    using Acc = typename Traits<S>::acc;
+    if (!p.ignore_done && *(volatile int *)&p.st->done)
+        return;
+    const long long b = blockIdx.x;
+    const long long row_begin = b * p.rows_base + (b < p.rows_rem ? b : (long long)p.rows_rem);
+    const int nrows = (int)(p.rows_base + (b < p.rows_rem ? 1 : 0));
+    map_body(MapForm<S, V, RG>{}, p, row_begin, nrows, static_cast<Acc *>(p.part_y) + b * p.ld,
+             p.part_stat + b, b == 0 ? p.skip_slot : -1);
+}
+
+struct MapFn {
+    template <int S, int V, int RG> static const void *get() { return (const void *)map_kernel<S, V, RG>; }
+};
+
+}  // namespace
 
 // --------------------------------------------------- Map, long rows --------
 //
@@ -1153,6 +1174,17 @@ cudaError_t cluster_prepare(int storage, int vpt, int rg, int C, size_t smem, in
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaOccupancyMaxActiveClusters(clusters, fn, &cfg);
+}
+
+cudaError_t team_map_prepare(int storage, int vpt, int rg) { return set_smem(dense_fn<MapFn>(storage, vpt, rg)); }
+
+cudaError_t team_launch(int storage, int vpt, int grid, size_t smem, cudaStream_t s, const MapArgs &a)
+{
+    const void *fn = dense_fn<MapFn>(storage, vpt, a.rows_per_slot);
+    if (!fn)
+        return cudaErrorInvalidValue;
+    void *args[] = {const_cast<MapArgs *>(&a)};
+    return cudaLaunchKernel(fn, dim3(grid), dim3(team_threads(a.teams, a.team_warps)), args, smem, s);
 }
 
 cudaError_t map_launch(int storage, int vpt, int grid, size_t smem, cudaStream_t s, const MapArgs &a)

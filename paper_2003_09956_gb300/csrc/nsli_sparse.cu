@@ -26,7 +26,7 @@
 // a row to finish (per-row counter) adds the slots (the block's threads in a
 // fixed tree), so the sums stay independent of timing.  Binary64 sums are
 // trees or independent running sums throughout: a dependent binary64
-// operation costs about 435 cycles on GB300.
+// operation costs about 300 cycles on a full GB300 SM (64 on an idle one).
 //
 // Small systems (x, y, the coefficients and a lambda / h table fit one CTA's
 // shared memory, the matrix its L1) run instead on sparse_resident_kernel:
@@ -68,7 +68,7 @@ template <typename T> __device__ __forceinline__ T warp_total(T v)
 }
 
 // Block sum in a fixed tree: warp butterflies, then a pairwise tree over the
-// 8 warp sums (GB300 takes about 435 cycles per dependent binary64 add, so
+// 8 warp sums (GB300 takes about 300 cycles per dependent binary64 add, so
 // every sum here is a tree rather than a chain).
 template <typename T> __device__ __forceinline__ T block_sum(T v, T *sh)
 {
@@ -681,8 +681,8 @@ __device__ __forceinline__ double res_fold(const double *part, int lane)
 // |v| as an integer that orders like |v| (the bits of a non-negative binary64)
 __device__ __forceinline__ long long abs_bits(double v) { return __double_as_longlong(v) & 0x7fffffffffffffffll; }
 
-// GB300 executes a dependent binary64 operation in about 435 cycles (a
-// measured chain of FMAs on one SM, against about 12 for binary32), so an
+// GB300 executes a dependent binary64 operation in 64 cycles with one warp on the
+// SM and about 300 with 16 (measured chains; binary32: about 12), so an
 // iteration's time is set by the depth of its binary64 dependency chain, and
 // the kernel is arranged to keep that chain short: rows longer than
 // kResLong go to warps of their own (lanes hold four partial sums added in a
