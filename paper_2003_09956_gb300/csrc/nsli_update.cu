@@ -256,6 +256,7 @@ template <int S, typename I, bool VEC> __device__ __forceinline__ void update_ro
     // pairs of nsli_sumsq.cuh); kUnroll loads in flight
     double n2 = 0.0;
     QuickSum<S != NSLI_FP8E4M3> quick;
+    quick_init(quick);
     for (I j0 = threadIdx.x; j0 < n; j0 += (I)kThreads * kUnroll) {
         if constexpr (S == NSLI_F64) {
             double v[kUnroll];
@@ -278,7 +279,7 @@ template <int S, typename I, bool VEC> __device__ __forceinline__ void update_ro
             // may take the value as it is)
 #pragma unroll
             for (int u = 0; u < kUnroll; u += 2)
-                quick.add(v[u], v[u + 1]);
+                quick_add(quick, v[u], v[u + 1]);
         }
     }
     if (bad)
