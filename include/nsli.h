@@ -86,9 +86,13 @@ typedef struct {
     int32_t stop;        /* NSLI_STOP_*                                             */
     double eps;          /* threshold of the stopping rule, >= 0                   */
     int64_t max_iter;    /* nsli_solve: maximum number of x-updates, >= 0           */
-    int32_t block_iters; /* iterations per captured CUDA graph (0: 32); for a small
-                            sparse system run on one CTA, iterations per launch
-                            (0: 1024)                                                */
+    int32_t block_iters; /* iterations per captured CUDA graph; for a small sparse
+                            system run on one CTA, iterations per launch.  0: the
+                            library chooses: dense rows that fit the registers go
+                            32 to 1024 iterations (about 64 GiB of A) per
+                            cooperative launch, other systems 32 per graph, small
+                            sparse ones 1024 per launch; while the handle's stream
+                            is being captured, launch by launch                     */
     int32_t reserved;    /* must be 0                                               */
     double rho;          /* translation per tick: b(k) = b0 + k * rho * Av          */
 } nsli_params;
