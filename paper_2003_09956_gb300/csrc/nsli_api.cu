@@ -715,9 +715,9 @@ int nsli_create(nsli_handle *out, int64_t m, int64_t n, int32_t storage, int32_t
     CKC(cudaMalloc(&h->part_y, (size_t)h->G * h->ld * accb), "allocate partial sums");
     CKC(cudaMalloc((void **)&h->part_stat, (size_t)h->G * sizeof(PartStat)), "allocate partial stats");
     CKC(cudaMalloc((void **)&h->rtab, (size_t)(m + 1) * 8), "allocate step table");
-    CKC(cudaMalloc((void **)&h->part_dx, (size_t)2 * h->red_grid * 8), "allocate step partials");
+    CKC(cudaMalloc((void **)&h->part_dx, (size_t)3 * h->red_grid * 8), "allocate step partials");
     CKC(cudaMalloc((void **)&h->iter_sync, 4 * sizeof(unsigned int)), "allocate grid counters");
-    CKC(cudaMalloc((void **)&h->iter_dmax, (size_t)h->red_grid * 8), "allocate step maxima");
+    CKC(cudaMalloc((void **)&h->iter_dmax, (size_t)2 * h->red_grid * 8), "allocate step maxima");
     CKC(cudaMalloc(&h->iter_stats, (size_t)2 * h->G * 32), "allocate iteration records");
     CKC(cudaMalloc((void **)&h->ybuf, (size_t)h->ld * 8), "allocate y");
     CKC(cudaMalloc((void **)&h->dtmp, (size_t)std::max<long long>(m, h->ld) * 8), "allocate staging");

@@ -2,6 +2,7 @@
 // rows (nsli_team.cuh; sm_103a): whole iterations in one launch, grouped Map
 // launches of a pool, and the persistent serving launch.
 #include "nsli_team.cuh"
+#include "nsli_handover.h"
 
 namespace nsli {
 
@@ -30,10 +31,12 @@ namespace {
 // -> 48 us), 32768 x 8192 bf16 116 -> 94 us, 131072 x 16384 binary32 1174 ->
 // 1159 us (the left figures with the one-team Map that the teams replace).
 // A: every CTA has written its partial sums and record.  C (ModAP): the
-// partial sums of ||y||^2.  B: the new x.  The records alternate between two
-// halves, since a CTA without columns to reduce does not hold up B.  Every
-// wait is bounded; a CTA that gives up raises the state's error flag, which
-// every waiting CTA watches.
+// partial sums of ||y||^2.  B: the new x.  The records (counts and maxima, dx^2
+// and max |dx_j|) alternate between two halves (nsli_handover.h), since a CTA
+// writes its next ones without waiting for the others' reads of the last, and
+// one without columns to reduce does not hold up B.  Every wait is bounded; a
+// CTA that gives up raises the state's error flag, which every waiting CTA
+// watches.
 struct IterShared {
     long long h;
     double mv, mn, mb, scale;
@@ -272,7 +275,7 @@ template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsume
                 ring_refill(p, src, q0, pend.slot, pend.stage);
             team_finish<S, V>(p, me, nbar, min(p.teams, src.ns), yr, stat, static_cast<Acc *>(p.part_y) + b * p.ld);
             if (tid == 0)
-                stats[(k & 1) * G + b] = stat;
+                stats[stat_half(k) * G + b] = stat;
         }
         // ---- A
         if (tid == 0) {
@@ -294,9 +297,10 @@ template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsume
         const Acc *py = static_cast<const Acc *>(r.part_y);
         group_sums<Acc>(py, p.ld, b, G, min(kIterBlocks, nmine) * 8, NW, part);
         if (warp == NW - 1) {
+            const int half = dx_half_read(k) * nblk;
             const bool rule_holds =
-                stop == NSLI_STOP_STEP && k > 0 && step_rule_holds(r.part_dx, a.dmax, nblk, eps, lane);
-            const RowStat<Acc> all = stats_of<Acc>(stats + (k & 1) * G, G, lane);
+                stop == NSLI_STOP_STEP && k > 0 && step_rule_holds(r.part_dx + half, a.dmax + half, nblk, eps, lane);
+            const RowStat<Acc> all = stats_of<Acc>(stats + stat_half(k) * G, G, lane);
             // the stop decision, by one thread: binary64 comparisons, which
             // would occupy the SM's binary64 pipe for each of its warps
             if (lane == 0) {
@@ -344,6 +348,10 @@ template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsume
         const double s = modap || h == 0 ? 0.0 : __ldg(r.rtab + h);
         int pend_blk = -1;      // a block whose partial dx^2 is still to be summed
         double pend_d = 0.0;
+        auto put_pending = [&]() {
+            const int q = dx_half_written(k) * nblk + pend_blk;
+            put_dx(pend_d, r.part_dx + q, a.dmax + q, lane);
+        };
         auto step_column = [&](long long j, double scale, double y, double xo) {
             const double xn = xo - scale * y;
             r.x64[j] = xn;
@@ -372,10 +380,10 @@ template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsume
                         r.ybuf[j] = y;
                     const double y2 = warp_sum(in ? y * y : 0.0);
                     if (lane == 0)
-                        r.part_dx[nblk + blk] = y2;
+                        r.part_dx[2 * nblk + blk] = y2;
                 } else {
                     if (pend_blk >= 0)
-                        put_dx(pend_d, r.part_dx + pend_blk, a.dmax + pend_blk, lane);
+                        put_pending();
                     pend_blk = blk;
                     pend_d = in ? step_column(j, s, y, xo) : 0.0;
                 }
@@ -394,7 +402,7 @@ template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsume
             if (!ok)
                 break;
             if (warp == 0)
-                modap_scale(r.part_dx + nblk, nblk, lambda, lane, &sh.mv, &sh.scale);
+                modap_scale(r.part_dx + 2 * nblk, nblk, lambda, lane, &sh.mv, &sh.scale);
             bar_threads(1, nbar);
             yn = sh.mv;
             if (warp < kIterBlocks)
@@ -402,7 +410,7 @@ template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsume
                 for (int blk = b + warp * G; blk < nblk; blk += kIterBlocks * G) {
                     const long long j = (long long)blk * kReduceCols + lane;
                     if (pend_blk >= 0)
-                        put_dx(pend_d, r.part_dx + pend_blk, a.dmax + pend_blk, lane);
+                        put_pending();
                     pend_blk = blk;
                     pend_d = j < p.ld ? step_column(j, sh.scale, r.ybuf[j], __ldcg(r.x64 + j)) : 0.0;   // (its own y)
                 }
@@ -422,7 +430,7 @@ template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsume
             *tk = (Acc)((double)tick * rho);
         }
         if (pend_blk >= 0)
-            put_dx(pend_d, r.part_dx + pend_blk, a.dmax + pend_blk, lane);
+            put_pending();
         bar_threads(1, nbar);
         ok = sh.ok != 0;
         if (!ok)
@@ -448,7 +456,7 @@ template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsume
     const int steps = k;   // made by this launch: iteration k was left before its step, or the loop ended
     double dx2 = 0.0;
     if (steps > 0) {
-        dx2 = fold_blocks(r.part_dx, nblk, lane);
+        dx2 = fold_blocks(r.part_dx + dx_half_written(steps - 1) * nblk, nblk, lane);
         if (!done && stop == NSLI_STOP_STEP && step_norm_below(dx2, eps)) {
             status = NSLI_OK;
             done = 1;

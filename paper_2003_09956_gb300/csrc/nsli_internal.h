@@ -121,9 +121,9 @@ struct ReduceArgs {
 // Whole iterations in one cooperative launch (nsli_dense.cu).
 struct IterArgs {
     MapArgs map;               // (part_stat is not used)
-    ReduceArgs red;            // part_dx: two halves of nblk sums (dx^2, y^2)
+    ReduceArgs red;            // part_dx: three parts of nblk sums (dx^2 in two halves, y^2)
     unsigned int *sync;        // grid counters: A, B, C, CTAs that have left
-    unsigned long long *dmax;  // nblk: max |dx_j| of a column block (bits)
+    unsigned long long *dmax;  // 2 x nblk: max |dx_j| of a column block (bits), in two halves
     void *stats;               // 2 x G records (32 bytes each at most)
     int iters, nblk;
 };
