@@ -2,7 +2,6 @@
 // rows (nsli_team.cuh; sm_103a): whole iterations in one launch, grouped Map
 // launches of a pool, and the persistent serving launch.
 #include "nsli_team.cuh"
-#include "nsli_handover.h"
 
 namespace nsli {
 
@@ -127,12 +126,14 @@ __device__ __noinline__ void modap_scale(const double *part, int nblk, double la
     }
 }
 
-// Counts and maxima over the CTAs' records (one warp; past L1, where the
-// records of two iterations ago may still be).
-template <typename Acc> __device__ __forceinline__ RowStat<Acc> stats_of(const RowStat<Acc> *rec, int G, int lane)
+// Counts (as 64 bits, to h) and maxima over the CTAs' records (one warp; past
+// L1, where the records of two iterations ago may still be).
+template <typename Acc>
+__device__ __forceinline__ RowStat<Acc> stats_of(const RowStat<Acc> *rec, int G, int lane, long long &h)
 {
     RowStat<Acc> s;
     s.clear();
+    h = 0;
     constexpr int U = sizeof(Acc) == 8 ? 1 : 5;   // (152 records: one round trip; binary64: 2218 us against 2253 at five)
 #pragma unroll 1
     for (int g0 = lane; g0 < G; g0 += 32 * U) {
@@ -150,10 +151,13 @@ template <typename Acc> __device__ __forceinline__ RowStat<Acc> stats_of(const R
             }
         }
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-            s.join(q[u]);
+        for (int u = 0; u < U; ++u) {
+            h += q[u].h;
+            s.join_maxima(q[u]);
+        }
     }
-    s.fold();
+    h = warp_count(h);
+    s.fold_maxima();
     return s;
 }
 
@@ -300,11 +304,12 @@ template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsume
             const int half = dx_half_read(k) * nblk;
             const bool rule_holds =
                 stop == NSLI_STOP_STEP && k > 0 && step_rule_holds(r.part_dx + half, a.dmax + half, nblk, eps, lane);
-            const RowStat<Acc> all = stats_of<Acc>(stats + stat_half(k) * G, G, lane);
+            long long violated;
+            const RowStat<Acc> all = stats_of<Acc>(stats + stat_half(k) * G, G, lane, violated);
             // the stop decision, by one thread: binary64 comparisons, which
             // would occupy the SM's binary64 pipe for each of its warps
             if (lane == 0) {
-                sh.h = all.h;
+                sh.h = violated;
                 sh.mv = Image<Acc>::back(all.mv);
                 sh.mn = Image<Acc>::back(all.mn);
                 sh.mb = Image<Acc>::back(all.mb);

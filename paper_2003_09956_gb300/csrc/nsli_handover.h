@@ -1,5 +1,6 @@
 // nsli_handover.h -- which words the iterations of one launch hand over in
-// (nsli_dense.cu): plain functions, also compiled for the host by the tests.
+// (nsli_dense.cu), and how row counts are summed over a warp: plain functions,
+// also compiled for the host by the tests.
 #pragma once
 
 #ifdef __CUDACC__
@@ -20,5 +21,20 @@ namespace nsli {
 NSLI_HD constexpr int stat_half(int k) { return k & 1; }             // the CTAs' counts and maxima of Map k
 NSLI_HD constexpr int dx_half_written(int k) { return k & 1; }       // dx of the step of iteration k
 NSLI_HD constexpr int dx_half_read(int k) { return (k - 1) & 1; }    // ... as read in iteration k >= 1
+
+// A count of rows in two parts whose sums over 32 lanes fit 32 bits, so that
+// two 32-bit warp reductions add counts of up to 2^53 rows a lane exactly (one
+// would wrap where more than 2^31 - 1 rows of a system are violated).
+struct CountParts {
+    unsigned int lo, hi;
+};
+NSLI_HD constexpr CountParts count_parts(long long h)
+{
+    return CountParts{(unsigned int)(h & 0x3ffffff), (unsigned int)(h >> 26)};
+}
+NSLI_HD constexpr long long count_join(unsigned int lo_sum, unsigned int hi_sum)
+{
+    return ((long long)hi_sum << 26) + (long long)lo_sum;
+}
 
 }  // namespace nsli

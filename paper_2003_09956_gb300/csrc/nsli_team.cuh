@@ -25,6 +25,7 @@
 // its bytes) is shared by enough rows or covered by other teams.
 #pragma once
 
+#include "nsli_handover.h"
 #include "nsli_map.cuh"
 
 #include <algorithm>
@@ -99,8 +100,10 @@ __device__ __forceinline__ void bar_threads(int id, int n)
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
-// Counts and maxima of some rows.  Binary64 maxima are kept as
-// order-preserving integers: exact, and quicker than binary64 comparisons.
+// Counts and maxima of some rows of one CTA (an int holds their number; over
+// the grid the counts are added as 64 bits: warp_count, stats_of).  Binary64
+// maxima are kept as order-preserving integers: exact, and quicker than
+// binary64 comparisons.
 template <typename Acc> struct Image;
 template <> struct Image<float> {
     using type = float;
@@ -114,6 +117,12 @@ template <> struct Image<double> {
     static __device__ __forceinline__ double back(unsigned long long v) { return red_ord_dec(v); }
     static __device__ __forceinline__ unsigned long long lowest() { return 0x000fffffffffffffull; }   // of -infinity
 };
+__device__ __forceinline__ long long warp_count(long long h)
+{
+    const CountParts c = count_parts(h);
+    const unsigned int lo = __reduce_add_sync(0xffffffffu, c.lo), hi = __reduce_add_sync(0xffffffffu, c.hi);
+    return count_join(lo, hi);
+}
 template <typename Acc> struct alignas(4 * sizeof(Acc)) RowStat {
     using I = typename Image<Acc>::type;
     typename std::conditional<sizeof(Acc) == 8, long long, int>::type h;
@@ -130,26 +139,25 @@ template <typename Acc> struct alignas(4 * sizeof(Acc)) RowStat {
         mn = up(mn, Image<Acc>::of(rn));
         mb = up(mb, Image<Acc>::of(ab));
     }
-    __device__ __forceinline__ void join(const RowStat &o)
+    __device__ __forceinline__ void join_maxima(const RowStat &o)
     {
-        h += o.h;
         mv = up(mv, o.mv);
         mn = up(mn, o.mn);
         mb = up(mb, o.mb);
     }
     // over the warp, in every lane: integer reductions of one instruction
     // instead of five shuffles and maxima each (exact; no value is a NaN: up()
-    // never takes one.  A lane's count is at most the rows of the warps or
-    // CTAs it joined; where it could pass 2^26 the 32 lanes' sum is taken as
-    // 64 bits)
+    // never takes one)
     __device__ __forceinline__ void fold()
     {
-        if constexpr (sizeof(Acc) == 8) {
-            const unsigned int lo = (unsigned int)(h & 0x3ffffff), hi = (unsigned int)(h >> 26);
-            h = ((long long)__reduce_add_sync(0xffffffffu, hi) << 26) + __reduce_add_sync(0xffffffffu, lo);
-        } else {
+        if constexpr (sizeof(Acc) == 8)
+            h = warp_count(h);
+        else
             h = __reduce_add_sync(0xffffffffu, h);
-        }
+        fold_maxima();
+    }
+    __device__ __forceinline__ void fold_maxima()
+    {
         mv = top(mv);
         mn = top(mn);
         mb = top(mb);

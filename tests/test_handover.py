@@ -1,4 +1,5 @@
-"""Hand-overs between the thread blocks of a one-launch run, without a GPU.
+"""Hand-overs between the thread blocks of a one-launch run, and the sums of
+their row counts, without a GPU.
 
 csrc/nsli_handover.h says which words an iteration writes and reads.  Here it
 is compiled for the host, and the order that the grid's counters give is
@@ -22,7 +23,17 @@ def words(tmp_path_factory):
     src.write_text('#include "nsli_handover.h"\n'
                    'extern "C" int stat_half(int k) { return nsli::stat_half(k); }\n'
                    'extern "C" int dx_half_written(int k) { return nsli::dx_half_written(k); }\n'
-                   'extern "C" int dx_half_read(int k) { return nsli::dx_half_read(k); }\n')
+                   'extern "C" int dx_half_read(int k) { return nsli::dx_half_read(k); }\n'
+                   '// 32 lanes added by two 32-bit reductions, as warp_count does\n'
+                   'extern "C" long long lanes_total(const long long *h) {\n'
+                   '    unsigned int lo = 0, hi = 0;\n'
+                   '    for (int i = 0; i < 32; ++i) {\n'
+                   '        const nsli::CountParts c = nsli::count_parts(h[i]);\n'
+                   '        lo += c.lo;\n'
+                   '        hi += c.hi;\n'
+                   '    }\n'
+                   '    return nsli::count_join(lo, hi);\n'
+                   '}\n')
     lib = d / "words.so"
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(src), "-o", str(lib)], check=True)
     return ctypes.CDLL(str(lib))
@@ -115,3 +126,13 @@ def test_one_half_for_dx_would_be_overwritten(words):
         dx_half_read = staticmethod(lambda k: 0)
     for modap, columns in ((False, (True, True)), (False, (True, False)), (True, (True, False))):
         assert faults(run_events(One, columns, 4, modap))
+
+
+@pytest.mark.parametrize("lanes", [[0] * 32, [1] * 32, [2 ** 26 - 1] * 32, [2 ** 26] * 32, [2 ** 31 - 1] * 32,
+                                   [2 ** 31] + [0] * 31, [2 ** 52 + 2 ** 26 - 1] * 32,
+                                   [(i * 0x9e3779b97f4a7c15) % 2 ** 40 for i in range(32)]])
+def test_counts_of_a_warp_add_exactly(words, lanes):
+    """Counts whose total leaves 32 bits (a system of more than 2^31 rows may
+    have them all violated; its total is the index of a table)."""
+    words.lanes_total.restype = ctypes.c_longlong
+    assert words.lanes_total((ctypes.c_longlong * 32)(*lanes)) == sum(lanes)
