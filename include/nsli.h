@@ -253,8 +253,11 @@ int nsli_get_norms2(nsli_handle h, double *out);
  * issues the bulk copy of its row slot `slot`, so its threads wait on a
  * barrier that nothing completes.  The bounded waits (about two seconds)
  * expire, the CTA records the timeout, waits (bounded) for its other copies
- * and returns.  Returns NSLI_ERR_TIMEOUT when detection works (NSLI_OK if
- * slot is beyond CTA 0's rows); the handle stays usable.  Synchronises. */
+ * and returns.  Then, where a run's iterations go in one launch, the same in
+ * such a launch (the other CTAs' waits for CTA 0 end too), and a launch after
+ * it, which leaves at once.  Returns NSLI_ERR_TIMEOUT when detection works
+ * (NSLI_OK if slot is beyond CTA 0's rows); the iterate is unchanged and the
+ * handle stays usable.  Synchronises. */
 int nsli_test_inject_timeout(nsli_handle h, int32_t slot);
 
 /* Progress of the last nsli_iterate / nsli_solve / sharded run (device

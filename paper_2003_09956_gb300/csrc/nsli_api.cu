@@ -429,10 +429,11 @@ int iterations_per_launch(const nsli_solver *h, const nsli_params *p)
     return (int)std::max<long long>(32, std::min<long long>(1024, (64ll << 30) / bytes));
 }
 
-cudaError_t launch_iterations(nsli_solver *h, int iters)
+cudaError_t launch_iterations(nsli_solver *h, int iters, int skip_slot = -1)
 {
     IterArgs a;
     a.map = map_args(h);
+    a.map.skip_slot = skip_slot;
     a.red = reduce_args(h);
     a.sync = h->iter_sync;
     a.dmax = h->iter_dmax;
@@ -1581,7 +1582,30 @@ int nsli_test_inject_timeout(nsli_handle h, int32_t slot)
     int rc = read_state(h);
     CK(cudaMemsetAsync(&h->st->error, 0, sizeof(int), h->stream), "clear error");
     CK(cudaStreamSynchronize(h->stream), "synchronize");
-    return rc;
+    if (!h->iter_ok || (rc != NSLI_OK && rc != NSLI_ERR_TIMEOUT))
+        return rc;
+    // the same in one launch of whole iterations (none of which may step),
+    // and a launch after it, which has to leave at once
+    DevState keep = *h->st_host;
+    keep.error = 0;
+    nsli_params p{};
+    p.lambda = 1.0;
+    int rc2 = begin_run(h, &p, NSLI_STOP_NONE, 0);
+    if (rc2 != NSLI_OK)
+        return rc2;
+    CK(launch_iterations(h, 2, slot), "launch iterations");
+    if (rc == NSLI_ERR_TIMEOUT) {
+        CK(launch_iterations(h, 2), "launch iterations");
+        h->launches += 1;
+    }
+    h->launches += 1;
+    rc2 = read_state(h);
+    if (rc2 == NSLI_ERR_TIMEOUT && (h->st_host->done || h->st_host->it))
+        rc2 = set_err(h, NSLI_ERR_CUDA, "a launch after an expired wait ran on");
+    CK(cudaMemcpyAsync(h->st, &keep, sizeof keep, cudaMemcpyHostToDevice, h->stream), "restore state");
+    CK(cudaMemsetAsync(h->iter_sync, 0, 4 * sizeof(unsigned int), h->stream), "clear grid counters");
+    CK(cudaStreamSynchronize(h->stream), "synchronize");
+    return rc2;
 }
 
 int nsli_get_stored_rows(nsli_handle h, int64_t row0, int64_t rows, double *out)

@@ -217,8 +217,12 @@ template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsume
     const MapArgs &p = a.map;
     const ReduceArgs &r = a.red;
     DevState *st = p.st;
-    if (*(volatile int *)&st->done)
-        return;   // the same for every CTA: the state changes after all have left
+    // the same for every CTA: the state changes after all have left.  Also
+    // after a launch that gave up, whose counters and records are unfinished
+    // until the next run begins (an error raised meanwhile by a CTA of this
+    // launch ends the others' waits too)
+    if (*(volatile int *)&st->done || *(volatile int *)&st->error)
+        return;
     extern __shared__ __align__(128) unsigned char smem[];
     IterShared &sh = *reinterpret_cast<IterShared *>(smem + kHIter);
     const int nbar = (int)blockDim.x, NW = nbar >> 5;
@@ -227,7 +231,7 @@ template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsume
     const long long row_begin = (long long)b * p.rows_base + min((long long)b, (long long)p.rows_rem);
     const int nrows = (int)(p.rows_base + (b < p.rows_rem ? 1 : 0));
     RowStat<Acc> *stats = static_cast<RowStat<Acc> *>(a.stats);
-    const RingSource src = ring_source(p, row_begin, nrows, a.iters, -1);
+    const RingSource src = ring_source(p, row_begin, nrows, a.iters, b == 0 ? p.skip_slot : -1);
     const bool resident = src.ns <= p.nstage;
     team_init(p, src);
 

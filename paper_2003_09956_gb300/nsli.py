@@ -476,8 +476,9 @@ class Solver:
         return out
 
     def inject_timeout(self, slot=1):
-        """Failure-detection test: returns the status of a Map launch whose
-        first CTA waits on a bulk copy that is never issued."""
+        """Failure-detection test: returns the status of a Map launch, and of
+        one of whole iterations, whose first CTA waits on a bulk copy that is
+        never issued."""
         return int(load().nsli_test_inject_timeout(self._h, int(slot)))
 
     def norms2(self):
