@@ -4,6 +4,8 @@
 // kernel from n and the storage type, captures blocks of iterations into
 // CUDA graphs, and runs the solve loop (graph block, read 64-byte state,
 // binary64 confirmation of candidate stops).
+#include <cudaTypedefs.h>
+
 #include <algorithm>
 #include <atomic>
 #include <climits>
@@ -17,6 +19,7 @@
 
 #include "nsli.h"
 #include "nsli_internal.h"
+#include "nsli_range.h"
 
 using namespace nsli;
 
@@ -507,9 +510,26 @@ cudaError_t alloc_flags(nsli_solver *h)
     return e;
 }
 
-// May a kernel of the handle read doubles at p directly?  (memory of its own
-// device, aligned; everything else goes through a staging copy)
-bool readable_by_kernel(const nsli_solver *h, const double *p)
+// The allocation that a device address lies in; false where the driver does
+// not know one.
+bool allocation_of(const void *p, CUdeviceptr *base, size_t *size)
+{
+    static const PFN_cuMemGetAddressRange_v3020 fn = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) !=
+                cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            f = nullptr;
+        return reinterpret_cast<PFN_cuMemGetAddressRange_v3020>(f);
+    }();
+    return fn && fn(base, size, (CUdeviceptr)(uintptr_t)p) == CUDA_SUCCESS;
+}
+
+// May a kernel of the handle read `count` doubles at p directly?  (memory of
+// its own device, aligned, and all of it inside the allocation; everything
+// else goes through a staging copy, which checks its own range)
+bool readable_by_kernel(const nsli_solver *h, const double *p, long long count)
 {
     cudaPointerAttributes at;
     if (reinterpret_cast<uintptr_t>(p) % 8 != 0)
@@ -518,7 +538,10 @@ bool readable_by_kernel(const nsli_solver *h, const double *p)
         cudaGetLastError();
         return false;
     }
-    return at.type == cudaMemoryTypeDevice && at.device == h->device;
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    return at.type == cudaMemoryTypeDevice && at.device == h->device && allocation_of(p, &base, &size) &&
+           range_covers(base, size, reinterpret_cast<uintptr_t>(p), (size_t)count, sizeof(double));
 }
 
 int read_flags(nsli_solver *h)
@@ -1195,7 +1218,7 @@ int nsli_update_b(nsli_handle h, const double *b0, int64_t tick)
         clear_flags(h);
         MetaArgs ma;
         // device memory: the record kernel reads it and keeps the copy
-        ma.b0_src = readable_by_kernel(h, b0) ? b0 : nullptr;
+        ma.b0_src = readable_by_kernel(h, b0, h->m) ? b0 : nullptr;
         if (!ma.b0_src)
             CK(cudaMemcpyAsync(h->b0_64, b0, (size_t)h->m * 8, cudaMemcpyDefault, h->stream), "copy b0");
         ma.b0_keep = h->b0_64;
@@ -1558,7 +1581,7 @@ int nsli_set_x(nsli_handle h, const double *x)
     if (!h || !x)
         return NSLI_ERR_ARG;
     clear_flags(h);
-    const bool direct = readable_by_kernel(h, x);
+    const bool direct = readable_by_kernel(h, x, h->n);
     if (!direct)
         CK(cudaMemcpyAsync(h->dtmp, x, (size_t)h->n * 8, cudaMemcpyDefault, h->stream), "copy x");
     CK(x_from_f64_launch(h->storage == NSLI_F64, h->stream, direct ? x : h->dtmp, h->x64, h->x, h->n, h->ld, h->flags),
