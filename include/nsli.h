@@ -89,7 +89,7 @@ typedef struct {
     int32_t block_iters; /* iterations per captured CUDA graph; for a small sparse
                             system run on one CTA, iterations per launch.  0: the
                             library chooses: dense rows that fit the registers go
-                            32 to 1024 iterations (about 64 GiB of A) per
+                            1 to 1024 iterations (up to 64 GiB of A) per
                             cooperative launch, other systems 32 per graph, small
                             sparse ones 1024 per launch; while the handle's stream
                             is being captured, launch by launch                     */

@@ -18,6 +18,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "nsli.h"
+#include "nsli_handover.h"
 #include "nsli_internal.h"
 #include "nsli_range.h"
 
@@ -418,9 +419,7 @@ cudaError_t launch_iteration(nsli_solver *h, int rule)
 
 // Iterations per launch of the one-launch form, 0 where it is not taken: the
 // caller asks for graphs of block_iters iterations, the rows are long or
-// sparse, or the stream is being captured.  A launch reads at most about 64
-// GB of A (some 10 ms), so that other streams get their turn and a solve its
-// polls; small systems take up to 1024 iterations.
+// sparse, or the stream is being captured.
 int iterations_per_launch(const nsli_solver *h, const nsli_params *p)
 {
     if (!h->iter_ok || p->block_iters > 0)
@@ -428,8 +427,7 @@ int iterations_per_launch(const nsli_solver *h, const nsli_params *p)
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
         return 0;
-    const long long bytes = h->m * (long long)h->row_bytes;
-    return (int)std::max<long long>(32, std::min<long long>(1024, (64ll << 30) / bytes));
+    return iterations_of(h->m * (long long)h->row_bytes);
 }
 
 cudaError_t launch_iterations(nsli_solver *h, int iters, int skip_slot = -1)

@@ -1,6 +1,6 @@
 // nsli_handover.h -- which words the iterations of one launch hand over in
-// (nsli_dense.cu), and how row counts are summed over a warp: plain functions,
-// also compiled for the host by the tests.
+// (nsli_dense.cu), how many there are, and how row counts are summed over a
+// warp: plain functions, also compiled for the host by the tests.
 #pragma once
 
 #ifdef __CUDACC__
@@ -21,6 +21,16 @@ namespace nsli {
 NSLI_HD constexpr int stat_half(int k) { return k & 1; }             // the CTAs' counts and maxima of Map k
 NSLI_HD constexpr int dx_half_written(int k) { return k & 1; }       // dx of the step of iteration k
 NSLI_HD constexpr int dx_half_read(int k) { return (k - 1) & 1; }    // ... as read in iteration k >= 1
+
+// Iterations per launch for a matrix of `bytes` bytes: at most 64 GiB of it are
+// read (some 10 ms) unless one iteration reads more, so that other streams get
+// their turn and a solve its polls; at most 1024.  (A launch's ring slots, of
+// 16 bytes or more and over two blocks or more, then number below 2^32.)
+NSLI_HD constexpr int iterations_of(long long bytes)
+{
+    const long long k = (64ll << 30) / bytes;
+    return (int)(k < 1 ? 1 : (k > 1024 ? 1024 : k));
+}
 
 // A count of rows in two parts whose sums over 32 lanes fit 32 bits, so that
 // two 32-bit warp reductions add counts of up to 2^53 rows a lane exactly (one

@@ -210,7 +210,7 @@ template <int S, int V> struct TeamThread {
 struct RingSource {
     const unsigned char *A, *meta;   // the block's first row and record
     int nrows, ns;
-    unsigned int total;              // (below 2^32: a launch reads at most some 64 GB)
+    unsigned int total;              // (below 2^32: iterations_of)
     int skip;                        // failure injection: this slot never arrives (-1: none)
 };
 __device__ __forceinline__ RingSource ring_source(const MapArgs &p, long long row_begin, int nrows, int passes, int skip)

@@ -24,6 +24,7 @@ def words(tmp_path_factory):
                    'extern "C" int stat_half(int k) { return nsli::stat_half(k); }\n'
                    'extern "C" int dx_half_written(int k) { return nsli::dx_half_written(k); }\n'
                    'extern "C" int dx_half_read(int k) { return nsli::dx_half_read(k); }\n'
+                   'extern "C" int iterations_of(long long b) { return nsli::iterations_of(b); }\n'
                    '// 32 lanes added by two 32-bit reductions, as warp_count does\n'
                    'extern "C" long long lanes_total(const long long *h) {\n'
                    '    unsigned int lo = 0, hi = 0;\n'
@@ -136,3 +137,16 @@ def test_counts_of_a_warp_add_exactly(words, lanes):
     have them all violated; its total is the index of a table)."""
     words.lanes_total.restype = ctypes.c_longlong
     assert words.lanes_total((ctypes.c_longlong * 32)(*lanes)) == sum(lanes)
+
+
+@pytest.mark.parametrize("log2", [4, 20, 26, 27, 30, 31, 32, 33, 35, 36, 37, 38])
+@pytest.mark.parametrize("off", [-16, 0, 16])
+def test_a_launch_reads_64_gib_at_most(words, log2, off):
+    """... unless one iteration reads more, so that a launch keeps the device
+    for some 10 ms."""
+    words.iterations_of.argtypes = [ctypes.c_longlong]
+    size = max(16, (1 << log2) + off)
+    k = words.iterations_of(size)
+    assert 1 <= k <= 1024
+    assert k == 1 or k * size <= 64 << 30
+    assert k == 1024 or (k + 1) * size > 64 << 30    # and no less than that allows
