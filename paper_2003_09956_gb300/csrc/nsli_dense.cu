@@ -82,7 +82,7 @@ __device__ __noinline__ double fold_blocks(const double *part, int nblk, int lan
 }
 
 // Does the step rule hold after the step whose dx the blocks' partials and
-// maxima describe?  (one warp; the sum only when no |dx_j| exceeds eps)
+// maxima describe?  (one warp; the sum only when no |dx_j| rules it out)
 __device__ __noinline__ bool step_rule_holds(const double *part_dx, const unsigned long long *dmax, int nblk, double eps,
                                              int lane)
 {
@@ -93,7 +93,7 @@ __device__ __noinline__ bool step_rule_holds(const double *part_dx, const unsign
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1)
         dm = max(dm, __shfl_xor_sync(0xffffffffu, dm, off));
-    if (__longlong_as_double((long long)dm) > eps * (1.0 + 1e-6))
+    if (__longlong_as_double((long long)dm) > step_gate(eps))
         return false;
     return step_norm_below(fold_blocks(part_dx, nblk, lane), eps);
 }

@@ -66,6 +66,15 @@ __host__ __device__ __forceinline__ bool step_norm_below(double dx2, double eps)
     return sqrt(dx2) < eps;
 }
 
+// A bound on |dx_j| above which ||dx|| < eps cannot hold (1e-6 of margin for
+// the sum's rounding), so that the sum need not be taken.  None where squares
+// of the size of eps^2 underflow: the root of the sum may then be 0 whatever
+// dx is.
+__host__ __device__ __forceinline__ double step_gate(double eps)
+{
+    return eps < 1e-150 ? 1.7976931348623157e308 : eps * (1.0 + 1e-6);
+}
+
 enum : int { ST_RUNNING = 2, ST_CANDIDATE = 3 };   // reported as NSLI_RUNNING / NSLI_CANDIDATE
 enum : int { ERRF_TIMEOUT = 1 };
 enum : int { PREPF_ZERO_ROW = 1, PREPF_NONFINITE = 2, PREPF_TIMEOUT = 4 };

@@ -772,9 +772,8 @@ __global__ void __launch_bounds__(kResThreads, 1) sparse_resident_kernel(const S
     // warps of their own for the long rows (columns), the last ones
     const int lw_r = min(NW / 2, p.n_res_long_rows), lw_c = min(NW / 2, p.n_res_long_cols);
     const int nt_r = (NW - lw_r) * 32, nt_c = (NW - lw_c) * 32;
-    // ||dx|| < eps is possible only if no |dx_j| exceeds eps (1e-6 of margin
-    // covers the rounding of the sum and the root)
-    const double gate = eps * (1.0 + 1e-6);
+    // the sum of dx^2 is taken only where no |dx_j| rules the step rule out
+    const double gate = step_gate(eps);
     int force = 0, status = 0, done = 0;
     long long it = 0, tick = 0, h_last = 0;
     double mv_last = 0, mn_last = 0, mb_last = 0, yn = 0;

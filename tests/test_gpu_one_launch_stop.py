@@ -72,3 +72,18 @@ def test_modap_step_is_lambda_long(storage, m, n):
             for g in got:
                 assert g[:2] == (status, iters)
                 np.testing.assert_array_equal(g[2], got[-1][2])
+
+
+@pytest.mark.parametrize("eps,iters", [(1e-100, 333), (1e-149, 495), (1e-151, 502), (1e-165, 538)])
+def test_step_rule_at_thresholds_whose_square_underflows(eps, iters):
+    """x <= 0 from x = 1 with half steps: step k is 2^-k long, its square 0
+    from k = 538 on.  ||dx|| is the root of the sum of squares in a one-launch
+    run too, and on one CTA."""
+    one = np.ones(1)
+    dense = nsli.Solver(np.ones((1, 1)), np.zeros(1), one, storage="f64")
+    sparse = nsli.SparseSolver(1, 1, np.array([0, 1]), np.array([0], np.int32), one, np.zeros(1), one, storage="f64")
+    with dense, sparse:
+        for s, block in ((dense, 0), (dense, 32), (sparse, 0), (sparse, 7)):
+            s.set_x(one)
+            r = s.solve(lam=0.5, stop="step", eps=eps, max_iter=1000, block_iters=block)
+            assert (r["status"], r["iters"], s.get_x()[0]) == (nsli.OK, iters, 2.0 ** -iters)
