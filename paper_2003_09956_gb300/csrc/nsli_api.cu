@@ -508,38 +508,36 @@ cudaError_t alloc_flags(nsli_solver *h)
     return e;
 }
 
-// The allocation that a device address lies in; false where the driver does
-// not know one.
-bool allocation_of(const void *p, CUdeviceptr *base, size_t *size)
+// May a kernel of the handle read `count` doubles at p directly?  (memory of
+// its own device, aligned, and all of it inside the allocation; everything
+// else goes through a staging copy, which checks its own range.  One driver
+// call for all of it: they are on the way of every new x and b.)
+bool readable_by_kernel(const nsli_solver *h, const double *p, long long count)
 {
-    static const PFN_cuMemGetAddressRange_v3020 fn = [] {
+    static const PFN_cuPointerGetAttributes_v7000 attributes = [] {
         void *f = nullptr;
         cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) !=
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) !=
                 cudaSuccess ||
             q != cudaDriverEntryPointSuccess)
             f = nullptr;
-        return reinterpret_cast<PFN_cuMemGetAddressRange_v3020>(f);
+        return reinterpret_cast<PFN_cuPointerGetAttributes_v7000>(f);
     }();
-    return fn && fn(base, size, (CUdeviceptr)(uintptr_t)p) == CUDA_SUCCESS;
-}
-
-// May a kernel of the handle read `count` doubles at p directly?  (memory of
-// its own device, aligned, and all of it inside the allocation; everything
-// else goes through a staging copy, which checks its own range)
-bool readable_by_kernel(const nsli_solver *h, const double *p, long long count)
-{
-    cudaPointerAttributes at;
-    if (reinterpret_cast<uintptr_t>(p) % 8 != 0)
+    const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+    if (!attributes || at % 8 != 0)
         return false;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
+    unsigned int type = 0, managed = 0;
+    int device = -1;
     CUdeviceptr base = 0;
     size_t size = 0;
-    return at.type == cudaMemoryTypeDevice && at.device == h->device && allocation_of(p, &base, &size) &&
-           range_covers(base, size, reinterpret_cast<uintptr_t>(p), (size_t)count, sizeof(double));
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                  CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *answers[] = {&type, &managed, &device, &base, &size};
+    if (attributes(5, what, answers, (CUdeviceptr)at) != CUDA_SUCCESS)
+        return false;
+    return type == CU_MEMORYTYPE_DEVICE && !managed && device == h->device &&
+           range_covers((uintptr_t)base, size, at, (size_t)count, sizeof(double));
 }
 
 int read_flags(nsli_solver *h)
