@@ -64,3 +64,26 @@ def test_every_entry_counts_once(storage, n):
             assert h == k == 1
             assert np.all(np.abs(y - want) <= TOL * np.abs(want))
             np.testing.assert_array_equal(y, z)
+
+
+@pytest.mark.parametrize("n", [1, 2, 255, 256, 257, 1793, 2047, 2048, 2049, 2305, 4099])
+def test_every_entry_counts_once_in_the_batched_form(n):
+    """The batched form's binary64 norms (eight entries per thread and step):
+    one violated row; y within 16 roundings of 2^-23 (1 / ||a||^2, the weight's
+    three bf16 terms and their products' sum), an entry's share 5e-5 or more."""
+    rng = np.random.default_rng(n)
+    m = 130
+    A = oracle.quantize_bf16(rng.uniform(0.5, 1.0, (m, n)).astype(np.float32))
+    A[:, 0] = 1.0
+    q = A[7].astype(np.float64)
+    assert (q * q).min() / np.dot(q, q) > 5e-5
+    b = np.full(m, 100.0)
+    b[7] = 1.0
+    X = np.zeros((2, n))
+    X[:, 0] = 2.0, 3.0
+    with nsli.BatchSolver(A, b, X) as s:
+        Y, h, _ = s.map_reduce()
+    for k in range(2):
+        want = (1.0 + k) * q / np.dot(q, q)
+        assert h[k] == 1
+        assert np.all(np.abs(Y[k] - want) <= 16 * 2.0 ** -23 * want)
