@@ -1232,8 +1232,19 @@ int nsli_update_b(nsli_handle h, const double *b0, int64_t tick)
         return read_flags(h);
     }
     if (tick >= 0) {
-        CK(set_tick_launch(h->stream, h->st, tick), "set tick");
-        h->launches += 1;
+        // A copy of eight bytes is quicker than a kernel (tick, then 2
+        // iterations of 2000 x 500 binary32, repeated: 25.2 against 27.1 us);
+        // its pageable source is staged before the call returns, but not
+        // where the stream is being captured: the kernel holds the value.
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        CK(cudaStreamIsCapturing(h->stream, &cs), "set tick");
+        if (cs == cudaStreamCaptureStatusNone) {
+            const long long t = tick;
+            CK(cudaMemcpyAsync(&h->st->tick, &t, sizeof t, cudaMemcpyHostToDevice, h->stream), "set tick");
+        } else {
+            CK(set_tick_launch(h->stream, h->st, tick), "set tick");
+            h->launches += 1;
+        }
     }
     return NSLI_OK;
 }
