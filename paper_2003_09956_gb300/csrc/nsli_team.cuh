@@ -333,9 +333,11 @@ __device__ __forceinline__ bool team_rows(const MapArgs &p, const TeamThread<S, 
     using Meta = typename Tr::meta;
     constexpr int EPV = Tr::EPV;
     constexpr int WL = 32 / RG;   // lanes per row in the folded reductions
-    // independent chains per row (binary64: one per vector and half, a tree
-    // after it: a dependent binary64 operation costs about 300 cycles)
-    constexpr int NCH = sizeof(Acc) == 8 ? V : ((V >= 4 && RG <= 2) ? 2 : 1);
+    // independent chains per row.  More of them do not pay in binary64 either:
+    // its pipe is the limit with many warps on the SM, and every chain is one
+    // more addition per thread and row (16385 x 8192 binary64, per iteration:
+    // a chain per vector 926 us, two chains 687 us)
+    constexpr int NCH = (V >= 4 && RG <= 2) ? 2 : 1;
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int R = RG;   // a slot is one row group
     const int W = p.team_warps, T = p.teams, lane = me.lane;
