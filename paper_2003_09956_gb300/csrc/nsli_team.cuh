@@ -336,7 +336,7 @@ __device__ __forceinline__ bool team_rows(const MapArgs &p, const TeamThread<S, 
     // independent chains per row.  More of them do not pay in binary64 either:
     // its pipe is the limit with many warps on the SM, and every chain is one
     // more addition per thread and row (16385 x 8192 binary64, per iteration:
-    // a chain per vector 926 us, two chains 687 us)
+    // a chain per vector 926 us, two chains 716 us)
     constexpr int NCH = (V >= 4 && RG <= 2) ? 2 : 1;
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int R = RG;   // a slot is one row group
