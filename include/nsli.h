@@ -90,9 +90,10 @@ typedef struct {
                             system run on one CTA, iterations per launch.  0: the
                             library chooses: dense rows that fit the registers go
                             1 to 1024 iterations (up to 64 GiB of A) per
-                            cooperative launch, other systems 32 per graph, small
-                            sparse ones 1024 per launch; while the handle's stream
-                            is being captured, launch by launch                     */
+                            cooperative launch, other systems (and a few rows of
+                            many columns) 32 per graph, small sparse ones 1024 per
+                            launch; while the handle's stream is being captured,
+                            launch by launch                                        */
     int32_t reserved;    /* must be 0                                               */
     double rho;          /* translation per tick: b(k) = b0 + k * rho * Av          */
 } nsli_params;

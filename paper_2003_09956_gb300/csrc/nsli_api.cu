@@ -419,10 +419,10 @@ cudaError_t launch_iteration(nsli_solver *h, int rule)
 
 // Iterations per launch of the one-launch form, 0 where it is not taken: the
 // caller asks for graphs of block_iters iterations, the rows are long or
-// sparse, or the stream is being captured.
+// sparse, few with many columns, or the stream is being captured.
 int iterations_per_launch(const nsli_solver *h, const nsli_params *p)
 {
-    if (!h->iter_ok || p->block_iters > 0)
+    if (!h->iter_ok || p->block_iters > 0 || !one_launch_pays(h->red_grid, h->G, h->storage == NSLI_F64))
         return 0;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)

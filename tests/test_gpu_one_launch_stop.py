@@ -30,7 +30,7 @@ def step_lengths(p, steps):
     return np.array(out)
 
 
-SHAPES = [("f32", 20, 8000), ("f64", 20, 4000), ("f32", 150, 8191), ("f32", 3000, 96), ("f64", 2432, 500),
+SHAPES = [("f32", 20, 8000), ("f32", 40, 8000), ("f64", 20, 4000), ("f32", 150, 8191), ("f32", 3000, 96), ("f64", 2432, 500),
           ("f32", 9001, 128), ("bf16", 500, 2048)]
 
 
@@ -57,7 +57,7 @@ def test_step_rule_stops_after_the_same_step(storage, m, n):
                 np.testing.assert_array_equal(g[4], got[-1][4])
 
 
-@pytest.mark.parametrize("storage,m,n", [("f32", 20, 8000), ("f32", 3000, 96)])
+@pytest.mark.parametrize("storage,m,n", [("f32", 20, 8000), ("f32", 40, 8000), ("f32", 3000, 96)])
 def test_modap_step_is_lambda_long(storage, m, n):
     """A ModAP step is lambda long: just above it the rule holds at once,
     just below it the run goes to its last iteration."""
