@@ -177,20 +177,28 @@ int choose_teams(nsli_solver *h, bool pooled)
     h->rows_base = h->m / h->G;
     h->rows_rem = (int)(h->m % h->G);
     const long long rows = h->rows_base + (h->rows_rem ? 1 : 0);
-    // One team with one vector per thread where a CTA's block is a group or
-    // two (up to 16 rows): the rows of a group go side by side anyway, and
-    // there are no teams' y to add (an iteration of 2000 x 500 binary32: 8.20
-    // us, with 16 one-warp teams 8.25 us).  Also short rows of a pool (below
-    // 2048 entries), whose items of hundreds of rows are summed row after row:
-    // the iterate of such a problem moves by 1 / n a step, so that another
-    // order of the sums would show in its tenth digit (1.3e-9 at n = 1024).
-    const bool one_team = h->nv <= kMapMaxConsumers && (rows <= 16 || (pooled && h->n < 2048));
+    // One team, as few vectors per thread as its warps need, where the rows of
+    // a CTA's block go side by side anyway and there would only be the teams' y
+    // to add.  With one vector per thread that is a block of a group or two (up
+    // to 16 rows; an iteration in one launch with one team against several:
+    // 2000 x 500 binary32 6.6 / 7.3 us, 2400 x 1024 binary32 7.1 / 8.5, 513 x 256
+    // binary64 8.4 / 9.4).  With more vectors, a block of one group (up to 4
+    // rows; Map and Reduce launches: 251 x 2500 binary32 13.2 / 14.5 us, 501 x
+    // 5000 14.6 / 16.5), but not in binary64, where the folds of more warps
+    // cost more than they save (205 x 2048: 20.6 / 19.1 us).
+    // Also short rows of a pool (below 2048 entries): several teams would be
+    // quicker (64 problems of 4096 x 1024 bf16: 370 us per round with one team,
+    // 208 with several) at the same error (9.5e-10 of the binary64 result
+    // either way), but the sums' order, and with it the tenth digit of served
+    // results, would change.
+    const bool one_group = !pooled && !f64 && rows <= 4;
+    const bool one_team = one_group || (h->nv <= kMapMaxConsumers && (rows <= 16 || (pooled && h->n < 2048)));
     // Otherwise as many vectors per thread as the registers hold (few warps
     // then share a row, and meet), fewer only where one warp holds the row
     // with them: a row takes team_warps warps, and the CTA's 16 mapping warps
     // hold as many teams as fit.
     h->vpt = 1;
-    while (!one_team && h->vpt < vlim && h->nv > 32 * h->vpt)
+    while (h->vpt < vlim && h->nv > (one_team ? kMapMaxConsumers : 32) * h->vpt)
         h->vpt *= 2;
     h->team_warps = (h->nv + 32 * h->vpt - 1) / (32 * h->vpt);
     h->teams = one_team ? 1 : (kMapMaxConsumers / 32) / h->team_warps;
@@ -209,7 +217,7 @@ int choose_teams(nsli_solver *h, bool pooled)
     auto stride_of = [&](int r) { return (int)round_up((long long)r * (h->row_bytes + 32), 128); };
     const int least = h->team_warps >= kLargeTeam ? 2 * h->teams + 1 : h->teams + 1;
     h->R = 1;
-    for (int r = one_team ? team_rg_max(1, f64) : std::min(4, team_rg_max(h->vpt, f64)); r > 1; r /= 2)
+    for (int r = one_team ? team_rg_max(h->vpt, f64) : std::min(4, team_rg_max(h->vpt, f64)); r > 1; r /= 2)
         if (budget / stride_of(r) >= least && (one_team || rows >= (long long)r * h->teams)) {
             h->R = r;
             break;
