@@ -279,7 +279,8 @@ template <int S, typename I, bool VEC> __device__ __forceinline__ void update_ro
             // may take the value as it is)
 #pragma unroll
             for (int u = 0; u < kUnroll; u += 2)
-                quick_add(quick, v[u], v[u + 1]);
+                if (j0 + (I)u * kThreads < n)   // (a pair of zeros would change nothing)
+                    quick_add(quick, v[u], v[u + 1]);
         }
     }
     if (bad)
@@ -345,14 +346,17 @@ template <int S, typename I, bool VEC> __device__ __forceinline__ void update_ro
     }
 }
 
-// Rows read from global memory (pass 2 finds them in L2).
-template <int S> __global__ void __launch_bounds__(kThreads) update_rows_kernel(const UpdateArgs p)
+// Rows read from global memory (pass 2 finds them in L2).  Bound by its loads'
+// latency: eight blocks share an SM (32 registers, indices of 32 bits where they
+// hold; with 40 registers six did: 2000 x 60000 binary32 rows 535 -> 424 us,
+// 200000 x 16 508 -> 416 us, 20000 x 4099 234 -> 193 us).
+template <int S, typename I> __global__ void __launch_bounds__(kThreads, 8) update_rows_kernel(const UpdateArgs p)
 {
     const long long r = blockIdx.x;
     if (r >= p.rows)
         return;
     const size_t eb = p.src_f64 ? 8 : 4;
-    update_row<S, long long, false>(p, r, static_cast<const unsigned char *>(p.src) + (size_t)r * (size_t)p.lda * eb);
+    update_row<S, I, false>(p, r, static_cast<const unsigned char *>(p.src) + (size_t)r * (size_t)p.lda * eb);
 }
 
 // Rows staged in shared memory by one bulk copy (the source row 16-byte
@@ -470,6 +474,18 @@ template <int S> cudaError_t staged_launch(unsigned grid, size_t smem, cudaStrea
     return cudaGetLastError();
 }
 
+template <typename I> cudaError_t global_launch(int storage, unsigned grid, cudaStream_t s, const UpdateArgs &a)
+{
+    switch (storage) {
+    case NSLI_F64: update_rows_kernel<NSLI_F64, I><<<grid, kThreads, 0, s>>>(a); break;
+    case NSLI_F32: update_rows_kernel<NSLI_F32, I><<<grid, kThreads, 0, s>>>(a); break;
+    case NSLI_BF16: update_rows_kernel<NSLI_BF16, I><<<grid, kThreads, 0, s>>>(a); break;
+    case NSLI_FP8E4M3: update_rows_kernel<NSLI_FP8E4M3, I><<<grid, kThreads, 0, s>>>(a); break;
+    default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
 // The staged kernel takes rows of up to this many source bytes (two blocks
 // per SM), whose start is 16-byte aligned on every row.
 constexpr size_t kStagedMaxBytes = 112 * 1024;
@@ -499,14 +515,8 @@ cudaError_t update_rows_launch(int storage, cudaStream_t s, const UpdateArgs &a)
         default: return cudaErrorInvalidValue;
         }
     }
-    switch (storage) {
-    case NSLI_F64: update_rows_kernel<NSLI_F64><<<grid, kThreads, 0, s>>>(a); break;
-    case NSLI_F32: update_rows_kernel<NSLI_F32><<<grid, kThreads, 0, s>>>(a); break;
-    case NSLI_BF16: update_rows_kernel<NSLI_BF16><<<grid, kThreads, 0, s>>>(a); break;
-    case NSLI_FP8E4M3: update_rows_kernel<NSLI_FP8E4M3><<<grid, kThreads, 0, s>>>(a); break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    // (32-bit indices within a row, a step past its end included)
+    return a.ld < (1ll << 30) ? global_launch<int>(storage, grid, s, a) : global_launch<long long>(storage, grid, s, a);
 }
 
 }  // namespace nsli
