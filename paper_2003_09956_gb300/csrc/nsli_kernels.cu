@@ -844,9 +844,10 @@ __global__ void __launch_bounds__(256) verify_kernel(const VerifyArgs p)
 // registers.  The binary64 norm takes eight entries per step, as many as it
 // folds into binary64 at once, so that it counts none: nsli_batch_create of
 // 65536 x 8192 with 64 problems 5.15 ms, against 6.0 ms one entry at a time
-// and 7.05 ms with four entries and a count.
+// and 7.05 ms with four entries and a count.  Binary64 storage: five blocks per
+// SM, four were slower (32768 x 16384: 6.85 -> 6.34 ms).
 template <int S, bool FAST>
-__global__ void __launch_bounds__(256, S == NSLI_F64 ? 4 : 6) prep_kernel(const PrepArgs p)
+__global__ void __launch_bounds__(256, S == NSLI_F64 ? 5 : 6) prep_kernel(const PrepArgs p)
 {
     const long long r = blockIdx.x;
     if (r >= p.rows)
@@ -951,9 +952,14 @@ __global__ void __launch_bounds__(256, S == NSLI_F64 ? 4 : 6) prep_kernel(const 
             for (int u = 0; u < U; ++u)
                 if (j0 + u * 256 < p.ld)
                     v[u] = put(j0 + u * 256, v[u]);
-            // (a zero past n changes neither sum)
+            if constexpr (!FAST)
+                if (j0 >= 256)
+                    sumsq_flush(sq);   // the step before; rows of one step need no binary64
+            // (a zero past n changes neither sum; two of them are left out)
 #pragma unroll
             for (int u = 0; u < U; u += 2) {
+                if (j0 + u * 256 >= p.n)
+                    break;
                 if constexpr (FAST) {
                     quick_add(sq, v[u], v[u + 1]);
                 } else {
@@ -961,8 +967,6 @@ __global__ void __launch_bounds__(256, S == NSLI_F64 ? 4 : 6) prep_kernel(const 
                     sumsq_add<0>(sq, v[u + 1]);
                 }
             }
-            if constexpr (!FAST)
-                sumsq_flush(sq);
         }
     }
     if (bad)
@@ -971,17 +975,7 @@ __global__ void __launch_bounds__(256, S == NSLI_F64 ? 4 : 6) prep_kernel(const 
     if constexpr (S != NSLI_F64) {
         __shared__ float2 spair[8];
         __shared__ double sacc[8];
-        if constexpr (FAST) {
-            t = sumsq_block_total<8>(sq, spair, sacc);   // (synchronises the block)
-        } else {
-            double v = warp_sum(sumsq_value(sq));
-            if (lane == 0)
-                sacc[wid] = v;
-            __syncthreads();
-            if (threadIdx.x == 0)
-                for (int q = 0; q < 8; ++q)
-                    t += sacc[q];
-        }
+        t = sumsq_block_total<8>(sq, spair, sacc);   // (synchronises the block)
     } else {
         n2 = warp_sum(n2);
         if (lane == 0)
