@@ -201,9 +201,9 @@ template <int S> __device__ __forceinline__ void store_row_vec(void *Arow, const
 }
 
 // The update of row r from its source row `src` (global or shared memory),
-// indices of type I within the row.
-template <int S, typename I, bool VEC> __device__ __forceinline__ void update_row(const UpdateArgs &p, long long r,
-                                                                                  const void *src)
+// indices of type I within the row.  SHORT: rows of half a step at most.
+template <int S, typename I, bool VEC, bool SHORT>
+__device__ __forceinline__ void update_row(const UpdateArgs &p, long long r, const void *src)
 {
     const long long gi = p.row0 + r;
     __shared__ double sred[kThreads / 32];
@@ -279,7 +279,7 @@ template <int S, typename I, bool VEC> __device__ __forceinline__ void update_ro
             // may take the value as it is)
 #pragma unroll
             for (int u = 0; u < kUnroll; u += 2)
-                if (j0 + (I)u * kThreads < n)   // (a pair of zeros would change nothing)
+                if (!SHORT || j0 + (I)u * kThreads < n)   // (a pair of zeros would change nothing)
                     quick_add(quick, v[u], v[u + 1]);
         }
     }
@@ -348,15 +348,16 @@ template <int S, typename I, bool VEC> __device__ __forceinline__ void update_ro
 
 // Rows read from global memory (pass 2 finds them in L2).  Bound by its loads'
 // latency: eight blocks share an SM (32 registers, indices of 32 bits where they
-// hold; with 40 registers six did: 2000 x 60000 binary32 rows 535 -> 424 us,
-// 200000 x 16 508 -> 416 us, 20000 x 4099 234 -> 193 us).
-template <int S, typename I> __global__ void __launch_bounds__(kThreads, 8) update_rows_kernel(const UpdateArgs p)
+// hold; with 40 registers six did: 2000 x 60000 binary32 rows 522 -> 419 us,
+// 200000 x 16 531 -> 410 us, 20000 x 4099 220 -> 185 us).
+template <int S, typename I, bool SHORT>
+__global__ void __launch_bounds__(kThreads, 8) update_rows_kernel(const UpdateArgs p)
 {
     const long long r = blockIdx.x;
     if (r >= p.rows)
         return;
     const size_t eb = p.src_f64 ? 8 : 4;
-    update_row<S, I, false>(p, r, static_cast<const unsigned char *>(p.src) + (size_t)r * (size_t)p.lda * eb);
+    update_row<S, I, false, SHORT>(p, r, static_cast<const unsigned char *>(p.src) + (size_t)r * (size_t)p.lda * eb);
 }
 
 // Rows staged in shared memory by one bulk copy (the source row 16-byte
@@ -392,7 +393,7 @@ template <int S> __global__ void __launch_bounds__(kThreads) update_rows_staged_
         }
         return;
     }
-    update_row<S, int, true>(p, r, srow);
+    update_row<S, int, true, false>(p, r, srow);
 }
 
 // Binary64-accurate ||a_i||^2 of stored rows, one block per row: the
@@ -474,13 +475,13 @@ template <int S> cudaError_t staged_launch(unsigned grid, size_t smem, cudaStrea
     return cudaGetLastError();
 }
 
-template <typename I> cudaError_t global_launch(int storage, unsigned grid, cudaStream_t s, const UpdateArgs &a)
+template <typename I, bool SHORT> cudaError_t global_launch(int storage, unsigned grid, cudaStream_t s, const UpdateArgs &a)
 {
     switch (storage) {
-    case NSLI_F64: update_rows_kernel<NSLI_F64, I><<<grid, kThreads, 0, s>>>(a); break;
-    case NSLI_F32: update_rows_kernel<NSLI_F32, I><<<grid, kThreads, 0, s>>>(a); break;
-    case NSLI_BF16: update_rows_kernel<NSLI_BF16, I><<<grid, kThreads, 0, s>>>(a); break;
-    case NSLI_FP8E4M3: update_rows_kernel<NSLI_FP8E4M3, I><<<grid, kThreads, 0, s>>>(a); break;
+    case NSLI_F64: update_rows_kernel<NSLI_F64, I, SHORT><<<grid, kThreads, 0, s>>>(a); break;
+    case NSLI_F32: update_rows_kernel<NSLI_F32, I, SHORT><<<grid, kThreads, 0, s>>>(a); break;
+    case NSLI_BF16: update_rows_kernel<NSLI_BF16, I, SHORT><<<grid, kThreads, 0, s>>>(a); break;
+    case NSLI_FP8E4M3: update_rows_kernel<NSLI_FP8E4M3, I, SHORT><<<grid, kThreads, 0, s>>>(a); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -515,8 +516,15 @@ cudaError_t update_rows_launch(int storage, cudaStream_t s, const UpdateArgs &a)
         default: return cudaErrorInvalidValue;
         }
     }
-    // (32-bit indices within a row, a step past its end included)
-    return a.ld < (1ll << 30) ? global_launch<int>(storage, grid, s, a) : global_launch<long long>(storage, grid, s, a);
+    // Rows of half a step (1024 entries) at most leave out the pairs of zeros
+    // past their end (all rows replaced, with and without: 50000 x 513 binary32
+    // 180 / 208 us, FP8 255 / 368; 20000 x 1000 101 / 111); longer ones do not
+    // look, which lets the step's sums run side by side (32768 x 16384 FP8 1020 /
+    // 999 us).  32-bit indices within a row, a step past its end included.
+    if (a.n <= kThreads * kUnroll / 2)
+        return global_launch<int, true>(storage, grid, s, a);
+    return a.ld < (1ll << 30) ? global_launch<int, false>(storage, grid, s, a)
+                              : global_launch<long long, false>(storage, grid, s, a);
 }
 
 }  // namespace nsli
