@@ -148,10 +148,12 @@ MAP_SOURCE_END = "// --------------------------------------------------- Map, lo
 def kernels_sha():
     """Hash of the source the Map kernel is compiled from: its barrier and
     bulk-copy helpers (nsli_async.cuh), the decode and Reduce helpers
-    (nsli_map.cuh), the Map body (nsli_team.cuh) and nsli_kernels.cu up to
-    the long-row section (the kernels after it do not enter the Map)."""
+    (nsli_map.cuh), the sums of row counts (nsli_handover.h), the Map body
+    (nsli_team.cuh) and nsli_kernels.cu up to the long-row section (the
+    kernels after it do not enter the Map)."""
     csrc = os.path.join(ROOT, "paper_2003_09956_gb300", "csrc")
-    helpers = "".join(open(os.path.join(csrc, f)).read() for f in ("nsli_async.cuh", "nsli_map.cuh", "nsli_team.cuh"))
+    helpers = "".join(open(os.path.join(csrc, f)).read() for f in ("nsli_async.cuh", "nsli_map.cuh", "nsli_handover.h",
+                                                                "nsli_team.cuh"))
     src = open(os.path.join(csrc, "nsli_kernels.cu")).read()
     end = src.find(MAP_SOURCE_END)
     return hashlib.sha256((helpers + src[:end if end >= 0 else len(src)]).encode()).hexdigest()[:12]

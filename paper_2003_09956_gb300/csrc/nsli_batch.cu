@@ -448,8 +448,9 @@ __global__ void finish_kernel(const float *Ypart, int splits, int Pp, long long 
                               int mode)
 {
     // one problem per block row: its lambda / h is one binary64 division per
-    // block, not one per thread (some 20 binary64 operations, which bound the
-    // kernel: 18 -> 8 us at 64 problems of n = 8192)
+    // block, not one per thread (some 20 binary64 operations, which bounded the
+    // kernel: 18.3 -> 11.8 us at 64 problems of n = 8192, each launch by itself
+    // and cold; a pass of eight iterations takes what it took, 3.64 ms)
     const long long p = blockIdx.y, j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     __shared__ double s_sh;
     if (mode != 2 && threadIdx.x == 0) {

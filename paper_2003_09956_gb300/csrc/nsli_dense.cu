@@ -24,11 +24,15 @@ namespace {
 //     exceeds eps.
 // What bounds it: large systems, HBM; small ones, the latencies of an
 // iteration's serial steps (x in, rows, y out, A, group sums, step, B: about 8
-// us where the rows take 1 us).  Measured per iteration, separate launches ->
-// here: 2000 x 500 binary32 16.8 -> 8.2 us, 513 x 256 binary64 19.4 -> 8.7 us,
-// 8192 x 2048 binary32 31.0 -> 14.8 us, 20011 x 4099 bf16 82 -> 44 us (ModAP 93
-// -> 48 us), 32768 x 8192 bf16 116 -> 94 us, 131072 x 16384 binary32 1174 ->
-// 1159 us (the left figures with the one-team Map that the teams replace).
+// us where the rows take 1 us).  Measured per iteration, graphs of 32 iterations
+// (Map and Reduce launches) -> here: 2000 x 500 binary32 12.3 -> 6.8 us, 513 x
+// 256 binary64 13.8 -> 8.4, 8192 x 2048 binary32 20.6 -> 14.4, 32768 x 4096 bf16
+// 58.8 -> 50.7, 65536 x 8192 bf16 179 -> 173, 131072 x 16384 binary32 1173 ->
+// 1165.  Not quicker where the Map is bound by its instructions and this
+// kernel, which keeps an iteration's progress beside the slices, has no
+// registers left: 131072 x 16384 bf16 616 -> 635, FP8 471 -> 505 (128 registers
+// and a spill, the Map kernel 120), 65536 x 8192 FP8 131 -> 133.  Those take it
+// all the same; block_iters gives the graphs.
 // A: every CTA has written its partial sums and record.  C (ModAP): the
 // partial sums of ||y||^2.  B: the new x.  The records (counts and maxima, dx^2
 // and max |dx_j|) alternate between two halves (nsli_handover.h), since a CTA

@@ -250,7 +250,7 @@ __device__ __forceinline__ void reduce_stats(const PartStat *ps, int G, SH &sh, 
 
 // Column block `blk` of `nblk` of one problem's reduce-and-step, by a block
 // of NGRP warps (NGRP groups of partial rows per column: 8 in the
-// reduce kernels, 16 in the persistent serving kernel).
+// reduce kernels, 2 in the persistent serving kernel).
 template <typename Acc, int NGRP = 8>
 __device__ __forceinline__ void reduce_body(const ReduceArgs &p, const int blk, const int nblk,
                                             ReduceSharedT<NGRP> &sh, const int tid, const int bar_id)
