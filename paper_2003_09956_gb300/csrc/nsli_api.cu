@@ -1638,7 +1638,7 @@ int nsli_test_inject_timeout(nsli_handle h, int32_t slot)
     }
     h->launches += 1;
     rc2 = read_state(h);
-    if (rc2 == NSLI_ERR_TIMEOUT && (h->st_host->done || h->st_host->it))
+    if (rc2 == NSLI_ERR_TIMEOUT && (h->st_host->status != ST_RUNNING || h->st_host->it))
         rc2 = set_err(h, NSLI_ERR_CUDA, "a launch after an expired wait ran on");
     CK(cudaMemcpyAsync(h->st, &keep, sizeof keep, cudaMemcpyHostToDevice, h->stream), "restore state");
     CK(cudaMemsetAsync(h->iter_sync, 0, 4 * sizeof(unsigned int), h->stream), "clear grid counters");

@@ -221,11 +221,10 @@ template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsume
     const MapArgs &p = a.map;
     const ReduceArgs &r = a.red;
     DevState *st = p.st;
-    // the same for every CTA: the state changes after all have left.  Also
-    // after a launch that gave up, whose counters and records are unfinished
-    // until the next run begins (an error raised meanwhile by a CTA of this
-    // launch ends the others' waits too)
-    if (*(volatile int *)&st->done || *(volatile int *)&st->error)
+    // the same for every CTA: the state changes after all have left, or when
+    // one gives up, long after they have come.  Also set by a launch that gave
+    // up, whose counters and records are unfinished until the next run begins.
+    if (*(volatile int *)&st->done)
         return;
     extern __shared__ __align__(128) unsigned char smem[];
     IterShared &sh = *reinterpret_cast<IterShared *>(smem + kHIter);
@@ -459,6 +458,7 @@ template <int S, int V, int RG> __global__ void __launch_bounds__(kMapMaxConsume
             last = atomicAdd(a.sync + 3, 1u) == (unsigned)G - 1u;
         } else {
             atomicOr(&st->error, ERRF_TIMEOUT);
+            *(volatile int *)&st->done = 1;   // launches behind this one leave at once
         }
         sh.last = last;
     }
