@@ -93,7 +93,9 @@ typedef struct {
                             cooperative launch, other systems (and a few rows of
                             many columns) 32 per graph, small sparse ones 1024 per
                             launch; while the handle's stream is being captured,
-                            launch by launch                                        */
+                            launch by launch.  Cooperative launches of several
+                            handles that do not fit the device together take
+                            turns; the kernels of graphs overlap                    */
     int32_t reserved;    /* must be 0                                               */
     double rho;          /* translation per tick: b(k) = b0 + k * rho * Av          */
 } nsli_params;
